@@ -133,7 +133,8 @@ int hg_set_temporal_depth(hg_grid* g, int k);
 int hg_set_temporal_exact(hg_grid* g, int exact);
 
 /* z planes per thread block of the single-sweep kernel (a tuning knob: more blocks and more z warm-up below, fewer
- * and longer blocks above); 0 restores the built-in rule.  Results do not depend on it. */
+ * and longer blocks above); 0 restores the built-in rule (under which a small grid's sub-step runs without z-marching
+ * blocks).  Results do not depend on it. */
 int hg_set_block_depth(hg_grid* g, int planes);
 
 /*

@@ -218,8 +218,34 @@ int cuda_fail(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return hg::cuda_fail(e_, what); \
     } while (0)
 
+// ---- programmatic dependent launch ----
+// The sub-steps of one grid are a chain of short launches, so a launch may start while its predecessor still runs: its
+// blocks become resident as the predecessor's last blocks leave room, set up, and wait (pdl_wait) until every write of
+// the predecessor is visible.  Every kernel launched this way waits before its first access to memory that another
+// kernel writes, and signals (pdl_trigger) at its start, since its successor waits by itself.  Both are no-ops in a
+// launch without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, const Args&... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&c, kernel, (KArgs)args...);
+    return e == cudaSuccess ? HG_OK : cuda_fail(e, "kernel launch");
+}
+
 // kernels' host launchers (each returns HG_OK or an error code)
-int launch_step_single(hg_grid* g);                  // one interior sweep: cur -> 1-cur (stencil.cu)
+int launch_step_single(hg_grid* g);                  // one sub-step: cur -> 1-cur, all ghosts (stencil.cu)
+int launch_step_small(hg_grid* g);                   // the same for a small grid (stencil_small.cu)
 int adjoint_inject(hg_grid* a, const void* v, int vdt);
 int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b);
 int adjoint_gradient(hg_grid* a, const void* acc_a, const void* acc_b, void* out, int odt, double* scratch);
@@ -255,8 +281,7 @@ int prof_fold(hg_grid* g);   // synchronise and add the recorded pairs to prof_m
 // ---- sweep arguments (stencil.cu) ----
 struct Bnd {
     int faces;              // 1: Robin ghosts to update (block epilogue)
-    int periodic;           // 1: copy the new boundary cells into the opposite ghosts (block epilogue)
-    int xfaces;             // 0, or HG_BC_PERIODIC: the x-face ghost copies are made inside the sweep loop
+    int periodic;           // 1: the sweep stores the new boundary cells into the opposite ghosts too
     int zskip;              // bit 0 / bit 1: the -z / +z face is an interface to a neighbouring slab (its ghost
                             // plane is supplied by the caller before each sub-step and never written by a sweep)
     const float2* robin32;  // (alpha, beta) per face ghost, compensated float grids

@@ -30,16 +30,15 @@ namespace hg {
 
 namespace {
 
-__device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpret_cast<const double2*>(p)); }
-__device__ __forceinline__ double2 ld2rw(const double* p) { return *reinterpret_cast<const double2*>(p); }
+__device__ __forceinline__ double2 ld2(const double* p) { return *reinterpret_cast<const double2*>(p); }
 __device__ __forceinline__ void st2(double* p, double2 v) { *reinterpret_cast<double2*>(p) = v; }
 
 
-// Boundary work rides in the same launch, after each block's z-march (so it adds no registers to the sweep).  Robin:
+// Boundary work of a batched FP64 entry rides in the same blocks, after each block's z-march.  Robin:
 // a block next to a face updates the face ghosts that border its own cells -- its rows and planes of an x face, its
 // x range and planes of a y face, its x range and rows of a z face -- to level n+1, from level-n values only (the
 // ghost and its interior neighbour), which no block of the launch writes.  Every face ghost belongs to exactly one
-// block.  Dirichlet ghosts are data.  Periodic: see block_periodic_copies.
+// block.  Dirichlet ghosts are data.  Periodic ghosts are stored with the cells they copy (faces.cuh).
 
 
 
@@ -112,16 +111,16 @@ struct DC {
     double v[C];
 };
 template <int C>
-__device__ __forceinline__ DC<C> ldd(const double* p, bool ro) {
+__device__ __forceinline__ DC<C> ldd(const double* p) {
     DC<C> r;
     if constexpr (C == 4) {
-        const double2 a = ro ? ld2(p) : ld2rw(p), b = ro ? ld2(p + 2) : ld2rw(p + 2);
+        const double2 a = ld2(p), b = ld2(p + 2);
         r.v[0] = a.x;
         r.v[1] = a.y;
         r.v[2] = b.x;
         r.v[3] = b.y;
     } else {
-        r.v[0] = ro ? __ldg(p) : *p;
+        r.v[0] = *p;
     }
     return r;
 }
@@ -130,9 +129,9 @@ __device__ __forceinline__ DC<C> ldd(const double* p, bool ro) {
 template <int WY, int C, bool UNIFORM>
 __device__ __forceinline__ void sweep_f64(const SweepArgs& A, int bx, int by, int bz) {
     constexpr int TW = 32 * C;
-    const double* __restrict__ phi_c = (const double*)A.hi_c;
-    double* __restrict__ phi_pn = (double*)A.hi_n;
-    const double* __restrict__ rho = (const double*)A.rho;
+    const double* phi_c = (const double*)A.hi_c;  // plain loads (dependent launch, see hg_internal.cuh)
+    double* phi_pn = (double*)A.hi_n;
+    const double* rho = (const double*)A.rho;
     const Layout& L = A.L;
     const Bnd& B = A.B;
     const double nu2 = A.nu2;
@@ -152,20 +151,20 @@ __device__ __forceinline__ void sweep_f64(const SweepArgs& A, int bx, int by, in
     long long q = L.at(i0, j, k0);
     DC<C> cm = zero, cc = zero;
     if (halo) {
-        cm = ldd<C>(phi_c + q - L.plane, true);
-        cc = ldd<C>(phi_c + q, true);
+        cm = ldd<C>(phi_c + q - L.plane);
+        cc = ldd<C>(phi_c + q);
     }
     for (int k = k0; k < k1; ++k, q += L.plane) {
         DC<C> cp = zero, ys = zero, yn = zero, pv = zero, r = zero;
         double xl = 0.0, xr = 0.0;
-        if (halo) cp = ldd<C>(phi_c + q + L.plane, true);
+        if (halo) cp = ldd<C>(phi_c + q + L.plane);
         if (active) {
-            ys = ldd<C>(phi_c + q - L.pitch, true);
-            yn = ldd<C>(phi_c + q + L.pitch, true);
-            pv = ldd<C>(phi_pn + q, false);
-            r = ldd<C>(rho + q, true);
-            if (lane == 0) xl = __ldg(phi_c + q - 1);
-            if (lane == 31 && i0 + C <= L.nx) xr = __ldg(phi_c + q + C);
+            ys = ldd<C>(phi_c + q - L.pitch);
+            yn = ldd<C>(phi_c + q + L.pitch);
+            pv = ldd<C>(phi_pn + q);
+            r = ldd<C>(rho + q);
+            if (lane == 0) xl = phi_c[q - 1];
+            if (lane == 31 && i0 + C <= L.nx) xr = phi_c[q + C];
         }
         double sl = __shfl_up_sync(0xffffffffu, cc.v[C - 1], 1);
         double sr = __shfl_down_sync(0xffffffffu, cc.v[0], 1);
@@ -188,6 +187,17 @@ __device__ __forceinline__ void sweep_f64(const SweepArgs& A, int bx, int by, in
                 for (int e = 0; e < C; ++e)
                     if (i0 + e < L.nx) phi_pn[q + e] = o.v[e];
             }
+            if (B.periodic) {
+#pragma unroll
+                for (int e = 0; e < C; ++e) {
+                    if (i0 + e >= L.nx) continue;
+                    auto put = [&](long long g) {
+                        if (idx_ok(g, 1, L.elems, B.err)) phi_pn[g] = o.v[e];
+                    };
+                    periodic_x_ghosts(L, i0 + e, q + e, put);
+                    periodic_yz_ghosts(L, j, k, q + e, put);
+                }
+            }
         }
         cm = cc;
         cc = cp;
@@ -202,21 +212,14 @@ __device__ __forceinline__ void sweep_f64(const SweepArgs& A, int bx, int by, in
                     a[u] = B.robin[3 * gb.t[u]];
                     rg[u] = B.robin[3 * gb.t[u] + 1];
                     ri[u] = B.robin[3 * gb.t[u] + 2];
-                    pg[u] = __ldg(phi_c + gb.qg[u]);
-                    pi[u] = __ldg(phi_c + gb.qi[u]);
+                    pg[u] = phi_c[gb.qg[u]];
+                    pi[u] = phi_c[gb.qi[u]];
                 }
 #pragma unroll
             for (int u = 0; u < kGB; ++u)
                 if (u < gb.n && idx_ok(gb.qg[u], 1, L.elems, B.err))
                     phi_pn[gb.qg[u]] = robin_update_f64(a[u], rg[u], ri[u], pg[u], pi[u]);
         }, TW);
-    if (B.periodic) {
-        __syncthreads();
-        block_periodic_copies(L, bx * TW, by * WY, WY, k0, k1, bx, by, A.gx, A.gy, block_tid(), block_nth(),
-                              [&](long long q, long long d) {
-                                  if (idx_ok(d, 1, L.elems, B.err)) phi_pn[d] = phi_pn[q];
-                              }, TW);
-    }
 }
 
 // UNIFORM: the FP64 forms chosen per warp (batched launches) or per lane (the single-grid sweep), cell.cuh
@@ -230,71 +233,13 @@ __device__ __forceinline__ void sweep_f64_any(const SweepArgs& A, int bx, int by
 
 constexpr int kWY = 8;
 
-// ---- boundary kernels of a single-grid sub-step (one thread per face ghost) ----
-// ghost t of the face-major enumeration -> padded indices of the ghost, of its interior neighbour, and of the
-// interior cell on the opposite face (the periodic source); 32-bit in-face arithmetic
-__device__ __forceinline__ void ghost_cells(const Layout& L, const Bnd& B, int t, long long& qg, long long& qi,
-                                            long long& qo) {
-    int f = 0, base = 0;
-#pragma unroll
-    for (int u = 1; u < 6; ++u)
-        if (t >= (int)B.off[u]) {
-            f = u;
-            base = (int)B.off[u];
-        }
-    const int r = t - base;
-    const int na = f < 2 ? L.ny : L.nx;
-    const int a = r % na, b = r / na;
-    switch (f) {
-        case 0: qg = L.at(-1, a, b); qi = qg + 1; qo = L.at(L.nx - 1, a, b); break;
-        case 1: qg = L.at(L.nx, a, b); qi = qg - 1; qo = L.at(0, a, b); break;
-        case 2: qg = L.at(a, -1, b); qi = qg + L.pitch; qo = L.at(a, L.ny - 1, b); break;
-        case 3: qg = L.at(a, L.ny, b); qi = qg - L.pitch; qo = L.at(a, 0, b); break;
-        case 4: qg = L.at(a, b, -1); qi = qg + L.plane; qo = L.at(a, b, L.nz - 1); break;
-        default: qg = L.at(a, b, L.nz); qi = qg - L.plane; qo = L.at(a, b, 0); break;
-    }
-}
-
-// Robin: ghosts of level n+1 from level n (runs before the sweep; the sweep neither reads nor writes them).  The
-// x faces (whose ghosts are strided in memory) are done by the compensated-float sweep itself, so for those grids
-// this kernel covers the y and z faces only (t0 = first y-face ghost).
-__global__ void __launch_bounds__(256) k_ghosts_robin(const SweepArgs A, int t0) {
-    const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int)A.B.off[6]) return;
-    if (((A.B.zskip & 1) && t >= (int)A.B.off[4] && t < (int)A.B.off[5]) || ((A.B.zskip & 2) && t >= (int)A.B.off[5]))
-        return;  // a slab interface: the caller supplies that ghost plane
-    long long qg, qi, qo;
-    ghost_cells(A.L, A.B, t, qg, qi, qo);
-    if (A.prec == HG_PREC_F32K) {
-        const float* hc = (const float*)A.hi_c;
-        const lo_t* lc = (const lo_t*)A.lo_c;
-        const float2 ab = A.B.robin32[t];
-        const float hg = __ldg(hc + qg), hi = __ldg(hc + qi);
-        float gh, gl;
-        robin_update_f32k(ab.x, ab.y, hg, lo_decode(hg, lc[qg]), hi, lo_decode(hi, lc[qi]), gh, gl);
-        if (!idx_ok(qg, 1, A.L.elems, A.B.err)) return;
-        ((float*)A.hi_n)[qg] = gh;
-        ((lo_t*)A.lo_n)[qg] = lo_encode(gh, gl);
-    } else {
-        const double* pc = (const double*)A.hi_c;
-        const double* R = A.B.robin;
-        if (!idx_ok(qg, 1, A.L.elems, A.B.err)) return;
-        ((double*)A.hi_n)[qg] = robin_update_f64(R[3 * t], R[3 * t + 1], R[3 * t + 2], __ldg(pc + qg), __ldg(pc + qi));
-    }
-}
-
-// periodic: ghosts of level n+1 are copies of the new values on the opposite face (runs after the sweep)
-__global__ void __launch_bounds__(256) k_ghosts_periodic(const SweepArgs A, int t0) {
-    const int t = t0 + blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= (int)A.B.off[6]) return;
-    long long qg, qi, qo;
-    ghost_cells(A.L, A.B, t, qg, qi, qo);
-    if (A.prec == HG_PREC_F32K) {
-        ((float*)A.hi_n)[qg] = ((const float*)A.hi_n)[qo];
-        ((lo_t*)A.lo_n)[qg] = ((const lo_t*)A.lo_n)[qo];
-    } else {
-        ((double*)A.hi_n)[qg] = ((const double*)A.hi_n)[qo];
-    }
+// Whether a single grid's sub-step runs as one thread per group of cells (stencil_small.cu).  The line lies where the
+// marching kernels overtake it (measured on cubes): compensated float 224^3 (60.7 against 61.2 us; 192^3 38.5 against
+// 45.6, 256^3 88 against 80), FP64 between 192^3 (107 against 131 us) and 256^3 (246 against 216).  A pinned block
+// depth (hg_set_block_depth) asks for the marching sweep.
+bool small_grid(const hg_grid* g) {
+    const long long n = (long long)g->nx * g->ny * g->nz;
+    return g->zb == 0 && n <= (g->prec == HG_PREC_F32K ? 11500000LL : 8000000LL);
 }
 
 int zchunk(const hg_grid* g) {
@@ -314,9 +259,19 @@ int zchunk(const hg_grid* g) {
     return zb;
 }
 
+// A single grid's FP64 sub-step.  Blocks with z index below nzb sweep; the further z slices hold the Robin ghosts, one
+// thread each (they depend on level n only).
 template <int WY>
-__global__ void __launch_bounds__(32 * WY, 2) k_step_f64(const SweepArgs A) {
-    sweep_f64_any<WY, false>(A, blockIdx.x, blockIdx.y, blockIdx.z);
+__global__ void __launch_bounds__(32 * WY, 2) k_step_f64(const SweepArgs A, int nzb) {
+    pdl_trigger();
+    pdl_wait();
+    if ((int)blockIdx.z < nzb) {
+        sweep_f64_any<WY, false>(A, blockIdx.x, blockIdx.y, blockIdx.z);
+    } else {
+        const long long b = ((long long)(blockIdx.z - nzb) * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+        const long long t = b * (32 * WY) + block_tid();
+        if (t < A.B.off[6]) robin_ghost(A, (int)t);
+    }
 }
 
 // entry of block b in a prefix table of n entries
@@ -413,7 +368,6 @@ SweepArgs sweep_args(const hg_grid* g, int zb, int cpl) {
     A.gy = (g->ny + kWY - 1) / kWY;
     A.B.faces = g->bc == HG_BC_ROBIN ? 1 : 0;
     A.B.periodic = g->bc == HG_BC_PERIODIC ? 1 : 0;
-    A.B.xfaces = 0;
     A.B.zskip = g->ziface;
     A.B.err = g->derr;
     A.B.robin32 = g->robin32;
@@ -424,40 +378,26 @@ SweepArgs sweep_args(const hg_grid* g, int zb, int cpl) {
 
 unsigned sweep_blocks(const SweepArgs& A) { return A.gx * A.gy * (unsigned)((A.L.nz + A.zb - 1) / A.zb); }
 
-// A single grid's sub-step: [Robin ghost kernel] -> sweep -> [periodic ghost kernel].
-// Compensated-float grids: the TMA-staged sweep writes all Robin ghosts of level n+1 (x/y faces by its producer
-// warp from the staged level-n values, z faces by the first and last chunk) and copies the periodic x-face ghosts;
-// the periodic kernel covers the y and z faces with coalesced accesses.  FP64 grids: all ghosts in the small
-// kernels.
+// A single grid's sub-step, one launch with every face ghost of the new level in it: the small-grid kernel, or the
+// TMA-staged sweep (Robin x/y faces by its producer warp, z faces by the first and last chunk), or the FP64 sweep
+// with its ghost blocks; periodic ghosts are stored with the cells they copy.
 int launch_step_single(hg_grid* g) {
+    if (small_grid(g)) return launch_step_small(g);
     SweepArgs A = sweep_args(g, g->zb);
-    const int robin = A.B.faces, periodic = A.B.periodic;
-    const bool f32k = g->prec == HG_PREC_F32K;
-    A.B.faces = 0;
-    A.B.periodic = 0;
-    if (f32k && periodic) A.B.xfaces = HG_BC_PERIODIC;
-    const int t0r = f32k ? (int)A.B.off[6] : 0;  // first ghost left to the Robin kernel (none for f32k)
-    const int t0p = f32k ? (int)A.B.off[2] : 0;  // first ghost left to the periodic kernel
-    if (robin && t0r < A.B.off[6]) {
-        k_ghosts_robin<<<(unsigned)((A.B.off[6] - t0r + 255) / 256), 256, 0, g->stream>>>(A, t0r);
-        HG_LAUNCHED("Robin ghost kernel");
-    }
     int rc = prof_begin(g);
     if (rc) return rc;
-    if (f32k) {
-        SweepArgs At = A;
-        At.B.faces = robin;  // x/y-face Robin ghosts by the producer warp
-        if ((rc = launch_sweep_f32k_tma(g, At))) return rc;
+    if (g->prec == HG_PREC_F32K) {
+        if ((rc = launch_sweep_f32k_tma(g, A))) return rc;
     } else {
-        k_step_f64<kWY><<<dim3(A.gx, A.gy, (g->nz + A.zb - 1) / A.zb), dim3(32, kWY), 0, g->stream>>>(A);
+        const int nzb = (g->nz + A.zb - 1) / A.zb;
+        const long long per_slice = (long long)A.gx * A.gy * 32 * kWY;
+        const int ghosts = A.B.faces ? (int)((A.B.off[6] + per_slice - 1) / per_slice) : 0;
+        A.B.faces = 0;  // not by the sweep blocks' epilogue
+        rc = launch_pdl(k_step_f64<kWY>, dim3(A.gx, A.gy, nzb + ghosts), dim3(32, kWY), 0, g->stream, A, nzb);
+        if (rc) return rc;
         HG_LAUNCHED("stencil sub-step kernel");
     }
-    if ((rc = prof_end(g))) return rc;
-    if (periodic) {
-        k_ghosts_periodic<<<(unsigned)((A.B.off[6] - t0p + 255) / 256), 256, 0, g->stream>>>(A, t0p);
-        HG_LAUNCHED("periodic ghost kernel");
-    }
-    return HG_OK;
+    return prof_end(g);
 }
 
 int launch_batch_class(cudaStream_t st, bool f64, const TmaEntry* tab, const unsigned* first, int n,

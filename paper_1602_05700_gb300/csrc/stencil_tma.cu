@@ -17,6 +17,7 @@ __global__ void __launch_bounds__(32 * (WY + 1), 3)
                     const SweepArgs A, int* err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[2 * S];
+    pdl_trigger();
     tma_sweep<WY, S>(&m_hi, &m_lo, &m_d, &m_s, A, blockIdx.x, blockIdx.y, blockIdx.z, err, smem, bars);
 }
 
@@ -100,14 +101,14 @@ int launch_sweep_f32k_tma(hg_grid* g, const SweepArgs& A) {
     SweepArgs At = A;
     At.gx = grid.x;
     At.gy = grid.y;
-    k_step_f32k_tma<kTmaWY, kStages><<<grid, 32 * (kTmaWY + 1), smem, g->stream>>>(
-        g->tm[0 + c], g->tm[2 + c], g->tm[4 + g->dcur], g->tm[6], At, g->derr);
+    rc = launch_pdl(k_step_f32k_tma<kTmaWY, kStages>, grid, dim3(32 * (kTmaWY + 1)), smem, g->stream, g->tm[0 + c],
+                    g->tm[2 + c], g->tm[4 + g->dcur], g->tm[6], At, g->derr);
+    if (rc) return rc;
     HG_LAUNCHED("TMA-staged sub-step kernel");
     return HG_OK;
 }
 
-// the batched-launch entry of grid g for its sub-step cur -> 1 - cur: Robin ghosts of all faces inside the launch,
-// periodic ghosts by the blocks' epilogue
+// the batched-launch entry of grid g for its sub-step cur -> 1 - cur: all ghosts inside the launch
 int tma_entry(hg_grid* g, TmaEntry* e, int zb) {
     int rc = tma_maps(g);
     if (rc) return rc;
@@ -119,7 +120,6 @@ int tma_entry(hg_grid* g, TmaEntry* e, int zb) {
     e->A = sweep_args(g, zb);
     e->A.gx = (g->nx + kTX - 1) / kTX;
     e->A.gy = (g->ny + kTmaWY - 1) / kTmaWY;
-    e->A.B.xfaces = 0;
     e->err = g->derr;
     return HG_OK;
 }

@@ -101,8 +101,7 @@ __device__ __forceinline__ uint2 ldsl4(const lo_t* p) { return *reinterpret_cast
 
 // The sweep of tile (bx, by) and z chunk bz of one grid by a block of 32 (WY + 1) threads (flat thread index),
 // with the stage ring in `smem` and 2 S mbarriers in `bars`.  m_hi .. m_s: tensor maps of hi, lo codes, dlt and s
-// of level n (kernel parameters or global memory).  With B.periodic set (batched launches) the consumers also copy
-// their tile's new boundary values into the periodic ghosts after the march.
+// of level n (kernel parameters or global memory).  Periodic ghosts are stored with the cells they copy.
 template <int WY, int S>
 __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtensorMap* m_lo, const CUtensorMap* m_d,
                                           const CUtensorMap* m_s, const SweepArgs& A, int bx, int by, int bz,
@@ -134,6 +133,7 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();  // single-grid launches start before the previous sub-step has ended; no effect in other launches
 
     if (warp == WY) {  // producer
         constexpr int lag = S - 1;  // face work trails the copies by this many planes
@@ -254,8 +254,8 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
     const int j = j0 + warp;
     const int i0 = x0 + lane * 4;
     const bool active = i0 < L.nx && j < L.ny;
-    const float* __restrict__ hi_c = (const float*)A.hi_c;
-    const lo_t* __restrict__ lo_c = (const lo_t*)A.lo_c;
+    const float* hi_c = (const float*)A.hi_c;  // plain loads: with dependent launch the level may still be written
+    const lo_t* lo_c = (const lo_t*)A.lo_c;     // when this kernel starts, which the read-only path does not allow
     float* __restrict__ hi_n = (float*)A.hi_n;
     lo_t* __restrict__ lo_n = (lo_t*)A.lo_n;
     float* __restrict__ dlt = (float*)A.dlt;
@@ -266,8 +266,8 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
     // plane k0 - 1 of the own row straight from global memory (it is not staged)
     float4 hm = z4, lm = z4;
     if (i0 <= L.nx && j < L.ny) {
-        hm = __ldg(reinterpret_cast<const float4*>(hi_c + q - L.plane));
-        lm = lo_decode4(hm, __ldg(reinterpret_cast<const uint2*>(lo_c + q - L.plane)));
+        hm = *reinterpret_cast<const float4*>(hi_c + q - L.plane);
+        lm = lo_decode4(hm, *reinterpret_cast<const uint2*>(lo_c + q - L.plane));
     }
     // a wait that gives up ends this warp's march, but not before the epilogue barrier (no thread is left waiting)
     bool ok = mbar_wait(smem_addr(&bar_full[0]), 0u, err);
@@ -315,7 +315,7 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_addr(&bar_empty[sc]));  // this warp is done with plane k's stage
         if (active)
-            group_update_store(L, B, nu2, i0, q, hc, lc, hl, ll, hr, lr, hs, hn, ls, ln, hm, hp, lm, lp, d, r,
+            group_update_store(L, B, nu2, i0, j, k0 + it, q, hc, lc, hl, ll, hr, lr, hs, hn, ls, ln, hm, hp, lm, lp, d, r,
                                hi_n, lo_n, dlt);
         hm = hc;
         hc = hp;
@@ -325,16 +325,6 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
     }
     if (ok && B.faces && k1 == L.nz && active && !(B.zskip & 2))
         zface(5, hc, lc, hm, lm, q);  // hc: plane nz, hm: plane nz - 1
-    if (B.periodic) {  // batched launches: periodic ghosts of the tile's boundary cells, after all consumers stored
-        asm volatile("bar.sync 1, %0;" ::"r"(32 * WY) : "memory");
-        if (ok)
-            block_periodic_copies(L, x0, j0, WY, k0, k1, bx, by, A.gx, A.gy, tid, 32 * WY,
-                                  [&](long long qs, long long qd) {
-                                      if (!idx_ok(qd, 1, L.elems, B.err)) return;
-                                      hi_n[qd] = hi_n[qs];
-                                      lo_n[qd] = lo_n[qs];
-                                  });
-    }
 }
 
 }  // namespace hg

@@ -358,8 +358,8 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     // level n at plane k0-2 (not staged), needed when plane k0-1 is an interior plane of an interior row
     if (R.in && k0 >= 1 && xa <= L.nx) {
         const long long q = L.at(xa, R.y, k0 - 2);
-        hm0 = __ldg(reinterpret_cast<const float4*>((const float*)A.hi_c + q));
-        lm0 = lo_decode4(hm0, __ldg(reinterpret_cast<const uint2*>((const lo_t*)A.lo_c + q)));
+        hm0 = *reinterpret_cast<const float4*>((const float*)A.hi_c + q);
+        lm0 = lo_decode4(hm0, *reinterpret_cast<const uint2*>((const lo_t*)A.lo_c + q));
     }
 
     for (int it = 0; it < iters; ++it) {
@@ -471,6 +471,8 @@ __global__ void __maxnreg__(96)  // 2 blocks of 320 threads per SM (5 warps of 9
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();
     const bool ragged = (int)(blockIdx.x * kFX) + kFX > A.L.nx;
     if (A.exact) {
         if (ragged)
@@ -516,12 +518,12 @@ int launch_temporal2_tma(hg_grid* g) {
     SweepArgs A = sweep_args(g, zb);
     A.B.faces = g->bc == HG_BC_ROBIN ? 1 : 0;
     A.B.periodic = 0;
-    A.B.xfaces = 0;
     const int c = g->cur;
     dim3 grid((g->nx + kFX - 1) / kFX, (g->ny + kFY - 1) / kFY, (g->nz + zb - 1) / zb);
     if ((rc = prof_begin(g))) return rc;
-    k_temporal2_tma<<<grid, kFThreads, F2::smem, g->stream>>>(g->tm2[0 + c], g->tm2[2 + c], g->tm2[4 + g->dcur],
-                                                              g->tm2[6], A, (float*)g->dlt[1 - g->dcur], g->derr);
+    if ((rc = launch_pdl(k_temporal2_tma, grid, dim3(kFThreads), F2::smem, g->stream, g->tm2[0 + c], g->tm2[2 + c],
+                         g->tm2[4 + g->dcur], g->tm2[6], A, (float*)g->dlt[1 - g->dcur], g->derr)))
+        return rc;
     HG_LAUNCHED("TMA-staged depth-2 sub-step kernel");
     return prof_end(g);
 }

@@ -1,0 +1,56 @@
+"""The small-grid sub-step (one thread per group of cells, all ghosts in one launch) against the z-marching sweeps, which a
+pinned block depth selects: the same arithmetic on the same values, so every cell and ghost must agree bit for bit,
+for rows shorter than a group, ragged rows, single rows and planes, every boundary condition and both precisions."""
+import numpy as np
+import pytest
+
+from paper_1602_05700_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+import paper_1602_05700_gb300 as hg  # noqa: E402
+from tests.test_gpu_parity import robin_cfl  # noqa: E402
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 2, 1), (4, 1, 9), (5, 7, 3), (33, 17, 10), (129, 9, 6), (64, 64, 20)])
+@pytest.mark.parametrize("bc", ["dirichlet", "robin", "periodic"])
+@pytest.mark.parametrize("prec", ["f32k", "f64"])
+def test_small_grid_equals_marching_sweep(prec, bc, shape):
+    nx, ny, nz = shape
+    h = 1.0 / 64
+    dt = (robin_cfl(nx, ny, nz, h) if bc == "robin" else 0.5) * h / np.sqrt(3.0)
+    rho = I.noise(shape[::-1], 301, 0.0, 2.0)
+    phi0 = I.noise(shape[::-1], 302, -1.0, -0.5)
+    prev0 = phi0 + 1e-3 * I.noise(shape[::-1], 303, -1.0, 1.0)
+    out = []
+    for depth in (0, 5):
+        g = hg.Grid(nx, ny, nz, h, (-0.5 * nx * h, -0.5 * ny * h, -0.5 * nz * h), 1.0, 1.0, dt, prec, bc)
+        g.set_block_depth(depth)
+        g.set_density(torch.from_numpy(rho).cuda())
+        g.set_phi(torch.from_numpy(phi0).cuda(), torch.from_numpy(prev0).cuda())
+        g.step(9)
+        g.set_block_depth(depth)
+        g.step(2)
+        out.append((g.phi_ghosted(), g.stats()["change_rel"]))
+        g.free()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert out[0][1] == out[1][1]
+
+
+@pytest.mark.parametrize("prec", ["f32k", "f64"])
+def test_small_slab_leaves_its_interface_ghosts_alone(prec):
+    """A slab's interface ghost planes are supplied by the caller: the ghost threads skip those faces."""
+    n, h = 12, 1.0 / 16
+    out = []
+    for depth in (0, 4):
+        g = hg.Grid(n, n, n, h, (-0.5 * n * h,) * 3, 1.0, 1.0, 0.25 * h, prec, "robin", z_interfaces=3)
+        g.set_block_depth(depth)
+        g.set_phi(torch.from_numpy(I.noise((n, n, n), 311, -1.0, -0.5)).cuda())
+        g.step(3)
+        out.append(g.phi_ghosted())
+        g.free()
+    assert np.array_equal(out[0], out[1])
