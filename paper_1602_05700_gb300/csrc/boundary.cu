@@ -12,10 +12,10 @@
 //                           phi_g^{n+1} = alpha phi_g^n + beta phi_i^n, alpha = 1 - nu/mu, beta = (nu/mu) r_i / r_g
 //                           (compensated float).  Its static limit r_g phi_g = r_i phi_i seeds a new state.  The
 //                           per-sub-step update is fused into the sweep kernels (stencil.cu, temporal.cu).
-//   Periodic                ghost = interior cell on the opposite face; the sweep kernels write these copies (in their
-//                           epilogue), the kernel here fills them for a freshly seeded state or an adjoint injection.
+//   Periodic                ghost = interior cell on the opposite face; the sweep kernels write these copies with the
+//                           cells, the kernel here fills them for a freshly seeded state or an adjoint injection.
 //
-// r^l Y_lm is evaluated as a polynomial (no trigonometry): with C_m + i S_m = (x + i y)^m,
+// The moments are in moments.cuh.  For the ghosts r^l Y_lm is evaluated as a polynomial (no trigonometry): with C_m + i S_m = (x + i y)^m,
 //   r^l Y_lm = n_lm q_l^m(z, r^2) {C_m (m > 0), 1 (m = 0), S_|m| (m < 0)},
 //   q_m^m = (-1)^m (2m-1)!!,  q_{m+1}^m = (2m+1) z q_m^m,
 //   q_l^m = ((2l-1) z q_{l-1}^m - (l+m-1) r^2 q_{l-2}^m) / (l - m),
@@ -27,6 +27,7 @@
 
 #include "cell.cuh"
 #include "hg_internal.cuh"
+#include "moments.cuh"
 
 namespace hg {
 
@@ -71,105 +72,6 @@ __device__ __forceinline__ void solid_harmonics(double x, double y, double z, co
                 R[base - m] = N.n[base + m] * q * S[m];
             }
         }
-    }
-}
-
-__device__ __forceinline__ double load_as_double(const void* p, int dtype, long long i) {
-    return dtype == HG_DT_F64 ? ((const double*)p)[i] : (double)((const float*)p)[i];
-}
-
-
-// ---- double-double sums of the moments -----------------------------------------------------------------------
-// Each moment is a sum over every cell (1.7e7 terms at 256^3).  A plain running or tree sum in FP64 carries a
-// rounding error that the lossless scheme then carries, through the Dirichlet data, into phi; so every partial sum
-// is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding errors), whose
-// error is of order n eps^2 of the sum of |terms|.  The final s + e, rounded once, is then the correctly rounded
-// sum of the terms except in the rare case that the exact sum lies within that tiny error of a midpoint between
-// two doubles.
-__device__ __forceinline__ void dd_add(double& s, double& e, double x) {
-    const double t = __dadd_rn(s, x);
-    const double v = __dsub_rn(t, s);
-    e = __dadd_rn(e, __dadd_rn(__dsub_rn(s, __dsub_rn(t, v)), __dsub_rn(x, v)));
-    s = t;
-}
-// (s, e) += (s2, e2), renormalised so that s is the rounded value of the pair
-__device__ __forceinline__ void dd_merge(double& s, double& e, double s2, double e2) {
-    dd_add(s, e, s2);
-    e = __dadd_rn(e, e2);
-    const double t = __dadd_rn(s, e);
-    e = __dsub_rn(e, __dsub_rn(t, s));
-    s = t;
-}
-__device__ __forceinline__ void dd_warp(double& s, double& e) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const double s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
-        dd_merge(s, e, s2, e2);
-    }
-}
-// block sum of one pair per thread (blockDim.x a multiple of 32, at most 1024); result valid in thread 0
-__device__ __forceinline__ void dd_block(double& s, double& e, double* sh) {
-    dd_warp(s, e);
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) {
-        sh[2 * w] = s;
-        sh[2 * w + 1] = e;
-    }
-    __syncthreads();
-    if (w == 0) {
-        const bool have = l < (int)(blockDim.x >> 5);
-        s = have ? sh[2 * l] : 0.0;
-        e = have ? sh[2 * l + 1] : 0.0;
-        dd_warp(s, e);
-    }
-}
-
-constexpr int kMomBlocks = 152;  // fixed, so that the result does not depend on the device
-
-template <int LMAX>
-__global__ void __launch_bounds__(kRedThreads) k_moments(const void* rho, int dtype, int nx, int ny, int nz, double h,
-                                                         double ox, double oy, double oz, YlmNorm N,
-                                                         double* partial) {
-    constexpr int NQ = (LMAX + 1) * (LMAX + 1);
-    __shared__ double sh[64];
-    double as[NQ], ae[NQ];
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) as[q] = ae[q] = 0.0;
-    const long long n = (long long)nx * ny * nz;
-    const double h3 = __dmul_rn(__dmul_rn(h, h), h);
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(c % nx);
-        const long long r = c / nx;
-        const int j = (int)(r % ny);
-        const int k = (int)(r / ny);
-        const double m = __dmul_rn(load_as_double(rho, dtype, c), h3);
-        if (m == 0.0) continue;
-        double R[NQ];
-        solid_harmonics<LMAX>(ox + (i + 0.5) * h, oy + (j + 0.5) * h, oz + (k + 0.5) * h, N, R);
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) dd_add(as[q], ae[q], __dmul_rn(m, R[q]));
-    }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double s = as[q], e = ae[q];
-        dd_block(s, e, sh);
-        if (threadIdx.x == 0) {
-            partial[2 * ((long long)blockIdx.x * NQ + q)] = s;
-            partial[2 * ((long long)blockIdx.x * NQ + q) + 1] = e;
-        }
-    }
-}
-
-// sum the pairs partial[2 (b nq + q) + {0, 1}] over b in a fixed order (one block); out[q] = the rounded pair
-__global__ void __launch_bounds__(kRedThreads) k_finish(const double* partial, int nblocks, int nq, double* out) {
-    __shared__ double sh[64];
-    for (int q = 0; q < nq; ++q) {
-        double s = 0.0, e = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x)
-            dd_merge(s, e, partial[2 * ((long long)b * nq + q)], partial[2 * ((long long)b * nq + q) + 1]);
-        dd_block(s, e, sh);
-        if (threadIdx.x == 0) out[q] = s;
     }
 }
 
@@ -275,12 +177,10 @@ __global__ void k_periodic(int prec, void* p, void* lo, Layout L, Faces F) {
 
 template <int LMAX>
 int run_moments(hg_grid* g, const void* rho, int dtype) {
-    constexpr int NQ = (LMAX + 1) * (LMAX + 1);
-    k_moments<LMAX><<<kMomBlocks, kRedThreads, 0, g->stream>>>(rho, dtype, g->nx, g->ny, g->nz, g->h, g->origin[0],
-                                                                g->origin[1], g->origin[2], g->ylm, g->red);
-    HG_LAUNCHED("multipole moment kernel");
-    k_finish<<<1, kRedThreads, 0, g->stream>>>(g->red, kMomBlocks, NQ, g->dres);
-    HG_LAUNCHED("moment finish kernel");
+    const cudaError_t e = launch_moments<LMAX>(rho, dtype, g->nx, g->ny, g->nz, g->h, g->origin, g->ylm, g->red, g->dres,
+                                               g->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "multipole moment kernels");
+    g->launches += 2;
     return HG_OK;
 }
 
@@ -443,16 +343,10 @@ int noalloc_scratch(double** out) {
 template <int LMAX>
 int noalloc_moments(const void* rho, int dtype, int nx, int ny, int nz, double h, const double* o, double* scratch,
                     double* Qdev, cudaStream_t st) {
-    constexpr int NQ = (LMAX + 1) * (LMAX + 1);
     YlmNorm N;
     fill_ylm_norms(N);
-    k_moments<LMAX><<<kMomBlocks, kRedThreads, 0, st>>>(rho, dtype, nx, ny, nz, h, o[0], o[1], o[2], N, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "multipole moment kernel");
-    k_finish<<<1, kRedThreads, 0, st>>>(scratch, kMomBlocks, NQ, Qdev);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "moment finish kernel");
-    return HG_OK;
+    const cudaError_t e = launch_moments<LMAX>(rho, dtype, nx, ny, nz, h, o, N, scratch, Qdev, st);
+    return e == cudaSuccess ? HG_OK : cuda_fail(e, "multipole moment kernels");
 }
 
 }  // namespace

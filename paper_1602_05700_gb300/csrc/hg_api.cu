@@ -46,10 +46,9 @@ void fill_ylm_norms(YlmNorm& N) {
     }
     for (int l = 0; l <= kMaxL; ++l)
         for (int m = 0; m <= l; ++m) {
-            double ratio = 1.0;  // (l-m)!/(l+m)!
-            for (int t = l - m + 1; t <= l + m; ++t) ratio /= (double)t;
-            double K = sqrt((2.0 * l + 1.0) / (4.0 * pi) * ratio);
-            N.n[l * l + l + m] = m == 0 ? K : sqrt(2.0) * K;
+            double prod = 1.0;  // (l+m)!/(l-m)!, exact (below 2^53 up to l = 8)
+            for (int t = l - m + 1; t <= l + m; ++t) prod *= (double)t;
+            N.n[l * l + l + m] = sqrt((2.0 * l + 1.0) / ((m == 0 ? 4.0 : 2.0) * prod * pi));
             if (l > m) N.inv_lm[l * l + l + m] = 1.0 / (double)(l - m);
         }
 }

@@ -1,0 +1,388 @@
+// FP64 multipole moments of a density, Q_lm = sum_cells rho h^3 r^l Y_lm(x) (arXiv 1602.05700, Sec. 4: Dirichlet boundary by
+// multipole expansion), by way of the Cartesian moments M_abc = sum rho X^a Y^b Z^c, a + b + c <= lmax.
+//
+// What bounds it: the FP64 pipe (2 lanes per SM and clock).  Evaluating the harmonics of every cell and adding each to
+// a double-double sum costs about 240 FP64 operations per cell at lmax = 4 (9.3 ms at 256^3, against 1.5 ms for the 20
+// sub-steps that follow).  r^l Y_lm is a homogeneous polynomial with integer coefficients up to one factor, so the sums can
+// be taken axis by axis and the harmonics formed once per block:
+//   * a lane owns a row (fixed j, k); 16 consecutive cells at a time it forms the local moments about their centre
+//     from sums and differences of mirrored cells (7 operations per pair at lmax = 4, the factors u^a being integers
+//     <= 15^8), shifts them to the grid's coordinates and adds them to the row's T_a (double-double): 6 per cell;
+//   * T_a times Z^c goes to the lane's sums over k (10 per row and (a, c)); Y^b, a transposing warp reduction (31 merges
+//     per 32 moments), the sum over warps and the change to Q_lm follow once per block.
+// Coordinates are in half cells about the grid's centre, X = 2 i + 1 - nx, so that every power is an exact integer and the
+// cancellation inside a harmonic (x^2 - y^2 of a round source) is exact.  All sums that cross a group of 16 cells are
+// double-double, and the Cartesian moments stay so through the shift to the origin and the change to Q_lm.
+// Lanes read rows of their own, 16 bytes at a time and a group ahead: the sectors are used whole out of L1, and 32
+// wavefronts per load are 13 us of the 256^3 launch, hidden under the FP64 work.  Float input becomes double by integer
+// instructions (exact), since conversions are slow as well; groups of zeros (vacuum around the source) are skipped.
+//
+// Measured (random density, us, harmonics per cell -> this): lmax 4: 32^3 155 -> 64, 128^3 1190 -> 102, 256^3 9316 ->
+// 361 (FP64 work alone: 220; the reduction and the change of basis are a fixed 60 of latency); lmax 8 at 256^3 30,000 ->
+// 848; lmax 0 at 256^3 350 -> 115.  Error against quad precision (largest over spheres, blobs, constants and noise,
+// centred and shifted origins, lmax 4 and 8, relative to the largest moment / to the largest of the same degree):
+// 3.2e-16 / 5.3e-15 -> 2.4e-16 / 1.6e-15.
+#pragma once
+
+#include "hg_internal.cuh"
+
+namespace hg {
+
+constexpr int kMomBlocks = 152;  // fixed, so that the result does not depend on the device
+constexpr int kMomWarps = 8;
+
+// number of monomials x^a y^b z^c with a + b + c < l, i.e. the index of the first one of degree l
+__host__ __device__ constexpr int mono_off(int l) { return l * (l + 1) * (l + 2) / 6; }
+// index of x^(l-b-c) y^b z^c among those of degree l
+__host__ __device__ constexpr int mono_at(int l, int b, int c) { return c * (l + 1) - c * (c - 1) / 2 + b; }
+constexpr int kMonoMax = (kMaxL + 1) * (kMaxL + 2) / 2;  // monomials of degree kMaxL
+
+// 2^l r^l Y_lm / n_lm as integer coefficients of the monomials of degree l:
+//   q_l^m = (-1)^m 2^-l sum_k (-1)^k (2l-2k)! / (k! (l-k)! (l-2k-m)!) z^(l-2k-m) (x^2 + y^2 + z^2)^k
+// (the expansion of the Legendre polynomial's m-th derivative) times C_m or S_m, C_m + i S_m = (x + i y)^m.
+struct HarmonicTable {
+    double c[kMaxQ][kMonoMax];
+};
+constexpr double cfact(int n) { return n < 2 ? 1.0 : n * cfact(n - 1); }
+constexpr double cbinom(int n, int k) { return cfact(n) / (cfact(k) * cfact(n - k)); }
+constexpr HarmonicTable make_harmonics() {
+    HarmonicTable T{};
+    for (int l = 0; l <= kMaxL; ++l)
+        for (int m = -l; m <= l; ++m) {
+            const int am = m < 0 ? -m : m;
+            for (int k = 0; 2 * k + am <= l; ++k) {
+                const double q = ((k + am) % 2 ? -1.0 : 1.0) * cfact(2 * l - 2 * k) /
+                                 (cfact(k) * cfact(l - k) * cfact(l - 2 * k - am));
+                for (int u = 0; u <= k; ++u)          // (x^2)^(k-u-v) (y^2)^u (z^2)^v
+                    for (int v = 0; u + v <= k; ++v)
+                        for (int p = m < 0 ? 1 : 0; p <= am; p += 2) {  // x^(am-p) y^p with i^p
+                            const double s = (p / 2) % 2 ? -1.0 : 1.0;
+                            T.c[l * l + l + m][mono_at(l, 2 * u + p, l - 2 * k - am + 2 * v)] +=
+                                q * s * cbinom(am, p) * cbinom(k, u) * cbinom(k - u, v);
+                        }
+            }
+        }
+    return T;
+}
+static __device__ const HarmonicTable kHarmonics = make_harmonics();
+
+// ---- double-double sums --------------------------------------------------------------------------------------
+// Each moment is a sum over every cell (1.7e7 terms at 256^3).  A plain running or tree sum in FP64 carries a
+// rounding error that the lossless scheme then carries, through the Dirichlet data, into phi; so every partial sum
+// is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding errors), whose
+// error is of order n eps^2 of the sum of |terms|.
+__device__ __forceinline__ void dd_add(double& s, double& e, double x) {
+    const double t = __dadd_rn(s, x);
+    const double v = __dsub_rn(t, s);
+    e = __dadd_rn(e, __dadd_rn(__dsub_rn(s, __dsub_rn(t, v)), __dsub_rn(x, v)));
+    s = t;
+}
+// (s, e) += (s2, e2), renormalised so that s is the rounded value of the pair
+__device__ __forceinline__ void dd_merge(double& s, double& e, double s2, double e2) {
+    dd_add(s, e, s2);
+    e = __dadd_rn(e, e2);
+    const double t = __dadd_rn(s, e);
+    e = __dsub_rn(e, __dsub_rn(t, s));
+    s = t;
+}
+// (s, e) += (a, ae) * (x, xe)
+__device__ __forceinline__ void dd_fma(double& s, double& e, double a, double ae, double x, double xe = 0.0) {
+    const double p = __dmul_rn(a, x);
+    const double pe = __fma_rn(a, xe, __fma_rn(ae, x, __fma_rn(a, x, -p)));
+    dd_add(s, e, p);
+    e = __dadd_rn(e, pe);
+}
+__device__ __forceinline__ void dd_warp(double& s, double& e) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double s2 = __shfl_xor_sync(0xffffffffu, s, o), e2 = __shfl_xor_sync(0xffffffffu, e, o);
+        dd_merge(s, e, s2, e2);
+    }
+}
+
+// a float as the double of the same value, without the FP64 conversion (normal values and zeros by shifts)
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned ex = (u >> 23) & 0xffu;
+    if (ex == 0xffu || (ex == 0u && (u << 1) != 0u)) return (double)x;
+    const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ bool nonzero(float x) { return (__float_as_uint(x) << 1) != 0u; }
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+
+constexpr int kMomGroup = 16;  // cells of a row taken together
+
+// the 16 cells of a row from cell `start` on; those before `lo` or beyond `hi` are 0.  vec: the row starts on a 16-byte
+// boundary and has a whole number of 16-byte words, so that a group inside it can be read in such words
+__device__ __forceinline__ void mom_load(const float* __restrict__ row, int start, int lo, int hi, bool vec,
+                                         float (&v)[kMomGroup]) {
+    if (vec && start >= 0 && start + kMomGroup <= hi) {
+#pragma unroll
+        for (int g = 0; g < kMomGroup; g += 4) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(row + start + g));
+            v[g] = x.x, v[g + 1] = x.y, v[g + 2] = x.z, v[g + 3] = x.w;
+        }
+        if (start < lo)
+#pragma unroll
+            for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo ? v[e] : 0.f;
+    } else {
+#pragma unroll
+        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo && start + e < hi ? __ldg(row + start + e) : 0.f;
+    }
+}
+__device__ __forceinline__ void mom_load(const double* __restrict__ row, int start, int lo, int hi, bool vec,
+                                         double (&v)[kMomGroup]) {
+    if (vec && start >= 0 && start + kMomGroup <= hi) {
+#pragma unroll
+        for (int g = 0; g < kMomGroup; g += 2) {
+            const double2 x = __ldg(reinterpret_cast<const double2*>(row + start + g));
+            v[g] = x.x, v[g + 1] = x.y;
+        }
+        if (start < lo)
+#pragma unroll
+            for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo ? v[e] : 0.0;
+    } else {
+#pragma unroll
+        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo && start + e < hi ? __ldg(row + start + e) : 0.0;
+    }
+}
+
+struct MomArgs {
+    int nx, ny, nz;
+    double h3[2];              // cell volume, as a pair
+    double off[3][2];          // offset of the grid's centre from the origin in half cells, as a pair, per axis
+    double hl[kMaxL + 1][2];   // (h / 4)^l as a pair: half cells and the table's 2^-l
+    int centred;               // off is zero
+};
+
+// per-block partial moments: partial[2 (block nq + q) + {0, 1}]
+template <typename T, int LMAX>
+__global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restrict__ rho, bool vec, MomArgs P,
+                                                               YlmNorm N, double* __restrict__ partial) {
+    constexpr int NQ = (LMAX + 1) * (LMAX + 1), NM = mono_off(LMAX + 1), NB = (NM + 31) / 32;
+    __shared__ double wm[kMomWarps][NB * 32][2], tot[NM][2], moved[NM][2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int m = lane; m < NB * 32; m += 32) wm[warp][m][0] = wm[warp][m][1] = 0.0;
+    // tasks: (32 rows, 1 plane), plane fastest; a warp takes a contiguous range, so that its rows stay the same
+    const long long tasks = (long long)((P.ny + 31) / 32) * P.nz, W = (long long)kMomBlocks * kMomWarps;
+    const long long w = (long long)blockIdx.x * kMomWarps + warp;
+    long long t = w * tasks / W;
+    const long long t1 = (w + 1) * tasks / W;
+    while (t < t1) {
+        const int jg = (int)(t / P.nz), k0 = (int)(t % P.nz);
+        const int k1 = (int)(t1 - t < P.nz - k0 ? k0 + (t1 - t) : P.nz);
+        t += k1 - k0;
+        const int j = jg * 32 + lane;
+        const bool mine = j < P.ny;
+        double As[LMAX + 1][LMAX + 1], Ae[LMAX + 1][LMAX + 1];  // [a][c], a + c <= LMAX
+#pragma unroll
+        for (int a = 0; a <= LMAX; ++a)
+#pragma unroll
+            for (int c = 0; c <= LMAX; ++c) As[a][c] = Ae[a][c] = 0.0;
+        for (int k = k0; k < k1; ++k) {
+            const T* row = rho + ((long long)k * P.ny + (mine ? j : 0)) * P.nx;
+            double Ts[LMAX + 1], Te[LMAX + 1];
+#pragma unroll
+            for (int a = 0; a <= LMAX; ++a) Ts[a] = Te[a] = 0.0;
+            // groups of 16 cells; the last one ends with the row (its cells that belong to the one before are masked), and
+            // a row shorter than a group sits in the group's middle: a group never reaches beyond the row, so its local
+            // powers are no larger than the row's own
+            const int ng = (P.nx + kMomGroup - 1) / kMomGroup, hi = mine ? P.nx : 0;
+            auto start_of = [&](int g) {
+                return g < ng - 1 ? g * kMomGroup : P.nx >= kMomGroup ? P.nx - kMomGroup : -((kMomGroup - P.nx) / 2);
+            };
+            T nv[kMomGroup];  // the next group's cells: in flight while this one is worked on
+            mom_load(row, start_of(0), 0, hi, vec, nv);
+            for (int g = 0; g < ng; ++g) {
+                const int i = start_of(g);
+                T v[kMomGroup];
+#pragma unroll
+                for (int e = 0; e < kMomGroup; ++e) v[e] = nv[e];
+                if (g + 1 < ng) mom_load(row, start_of(g + 1), (g + 1) * kMomGroup, hi, vec, nv);
+                bool any = false;
+#pragma unroll
+                for (int e = 0; e < kMomGroup; ++e) any = any || nonzero(v[e]);
+                if (!__any_sync(0xffffffffu, any)) continue;
+                double loc[LMAX + 1];
+#pragma unroll
+                for (int a = 0; a <= LMAX; ++a) loc[a] = 0.0;
+#pragma unroll
+                for (int p = 0; p < kMomGroup / 2; ++p) {  // the cells at -u and +u half cells from the group's centre
+                    const double u = kMomGroup - 1 - 2 * p;
+                    const double lo = widen(v[p]), hi = widen(v[kMomGroup - 1 - p]);
+                    const double s = __dadd_rn(lo, hi);
+                    const double d = LMAX ? __dsub_rn(hi, lo) : 0.0;
+                    double f = 1.0;
+#pragma unroll
+                    for (int a = 0; a <= LMAX; ++a) {
+                        loc[a] = __fma_rn((a & 1) ? d : s, f, loc[a]);
+                        f *= u;
+                    }
+                }
+                // about the group's centre -> the grid's coordinates: loc_a <- sum_b C(a, b) X^(a-b) loc_b
+                const double X = (double)(2 * i + kMomGroup - P.nx);
+#pragma unroll
+                for (int b = 1; b <= LMAX; ++b)
+#pragma unroll
+                    for (int a = LMAX; a >= b; --a) loc[a] = __fma_rn(X, loc[a - 1], loc[a]);
+#pragma unroll
+                for (int a = 0; a <= LMAX; ++a) dd_add(Ts[a], Te[a], loc[a]);
+            }
+            const double Z = (double)(2 * k + 1 - P.nz);
+            double zc = 1.0;
+#pragma unroll
+            for (int c = 0; c <= LMAX; ++c) {
+#pragma unroll
+                for (int a = 0; a + c <= LMAX; ++a) dd_fma(As[a][c], Ae[a][c], Ts[a], Te[a], zc);
+                zc *= Z;
+            }
+        }
+        // times Y^b, summed over the warp's rows: each step halves the lanes a moment is spread over and the moments a
+        // lane holds, so lane n ends with moment n of the batch
+        if constexpr (NM == 1) {
+            dd_warp(As[0][0], Ae[0][0]);
+            if (lane == 0) dd_merge(wm[warp][0][0], wm[warp][0][1], As[0][0], Ae[0][0]);
+            continue;
+        }
+        const double Y = (double)(2 * j + 1 - P.ny);
+        double yb[LMAX + 1];
+        yb[0] = 1.0;
+#pragma unroll
+        for (int b = 1; b <= LMAX; ++b) yb[b] = yb[b - 1] * Y;
+#pragma unroll
+        for (int B = 0; B < NB; ++B) {
+            double vs[32], ve[32];
+#pragma unroll
+            for (int n = 0; n < 32; ++n) vs[n] = ve[n] = 0.0;
+#pragma unroll
+            for (int l = 0; l <= LMAX; ++l)
+#pragma unroll
+                for (int c = 0; c <= l; ++c)
+#pragma unroll
+                    for (int b = 0; b + c <= l; ++b) {
+                        const int n = mono_off(l) + mono_at(l, b, c) - 32 * B;
+                        if (n >= 0 && n < 32) dd_fma(vs[n], ve[n], As[l - b - c][c], Ae[l - b - c][c], yb[b]);
+                    }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const bool up = lane & o;
+#pragma unroll
+                for (int n = 0; n < o; ++n) {
+                    const double s2 = __shfl_xor_sync(0xffffffffu, up ? vs[n] : vs[n + o], o);
+                    const double e2 = __shfl_xor_sync(0xffffffffu, up ? ve[n] : ve[n + o], o);
+                    if (up) {
+                        vs[n] = vs[n + o];
+                        ve[n] = ve[n + o];
+                    }
+                    dd_merge(vs[n], ve[n], s2, e2);
+                }
+            }
+            dd_merge(wm[warp][32 * B + lane][0], wm[warp][32 * B + lane][1], vs[0], ve[0]);
+        }
+    }
+    __syncthreads();
+    for (int m = threadIdx.x; m < NM; m += 32 * kMomWarps) {
+        double s = wm[0][m][0], e = wm[0][m][1];
+        for (int v = 1; v < kMomWarps; ++v) dd_merge(s, e, wm[v][m][0], wm[v][m][1]);
+        tot[m][0] = s;
+        tot[m][1] = e;
+    }
+    __syncthreads();
+    if (!P.centred) {  // about the grid's centre -> about the origin, one axis after the other (binomials)
+        for (int axis = 0; axis < 3; ++axis) {
+            for (int m = threadIdx.x; m < NM; m += 32 * kMomWarps) {
+                int l = 0, b = m, c = 0;
+                while (mono_off(l + 1) <= m) ++l;
+                for (b = m - mono_off(l); b > l - c; ++c) b -= l - c + 1;
+                const int pw = axis == 0 ? l - b - c : axis == 1 ? b : c;  // the power of this axis
+                double s = 0.0, e = 0.0, f = 1.0, fe = 0.0;               // binomial(pw, r) offset^r
+                for (int r = 0; r <= pw; ++r) {
+                    const int n = mono_off(l - r) + mono_at(l - r, b - (axis == 1 ? r : 0), c - (axis == 2 ? r : 0));
+                    dd_fma(s, e, tot[n][0], tot[n][1], f, fe);
+                    double g = 0.0, ge = 0.0;
+                    dd_fma(g, ge, f, fe, P.off[axis][0], P.off[axis][1]);
+                    const double n1 = (double)(pw - r), d = (double)(r + 1), gn = __dmul_rn(g, n1);
+                    f = __ddiv_rn(gn, d);
+                    fe = __ddiv_rn(__fma_rn(-f, d, gn) + __fma_rn(ge, n1, __fma_rn(g, n1, -gn)), d);
+                }
+                moved[m][0] = s;
+                moved[m][1] = e;
+            }
+            __syncthreads();
+            for (int m = threadIdx.x; m < NM; m += 32 * kMomWarps) {
+                tot[m][0] = moved[m][0];
+                tot[m][1] = moved[m][1];
+            }
+            __syncthreads();
+        }
+    }
+    for (int q = threadIdx.x; q < NQ; q += 32 * kMomWarps) {
+        int l = 0;
+        while ((l + 1) * (l + 1) <= q) ++l;
+        const int m = q - l * l - l;
+        double s = 0.0, e = 0.0;
+        for (int n = 0; n < (l + 1) * (l + 2) / 2; ++n) {
+            const double c = kHarmonics.c[q][n];
+            if (c != 0.0) dd_fma(s, e, tot[mono_off(l) + n][0], tot[mono_off(l) + n][1], c);
+        }
+        double vs = 0.0, ve = 0.0, us = 0.0, ue = 0.0, qs = 0.0, qe = 0.0;
+        dd_fma(vs, ve, s, e, P.hl[l][0], P.hl[l][1]);
+        dd_fma(us, ue, vs, ve, P.h3[0], P.h3[1]);
+        dd_fma(qs, qe, us, ue, N.n[l * l + l + (m < 0 ? -m : m)]);
+        partial[2 * ((long long)blockIdx.x * NQ + q)] = qs;
+        partial[2 * ((long long)blockIdx.x * NQ + q) + 1] = qe;
+    }
+}
+
+// one warp per moment: the pairs partial[2 (b nq + q) + {0, 1}] over the blocks b in a fixed order; out[q] = the
+// rounded pair (one block over all moments took 166 us at lmax = 4, a serial chain of FP64 latencies; this 5)
+__global__ void __launch_bounds__(32) k_finish_moments(const double* __restrict__ partial, int nq, double* __restrict__ out) {
+    double s = 0.0, e = 0.0;
+    for (int b = threadIdx.x; b < kMomBlocks; b += 32)
+        dd_merge(s, e, partial[2 * ((long long)b * nq + blockIdx.x)], partial[2 * ((long long)b * nq + blockIdx.x) + 1]);
+    dd_warp(s, e);
+    if (threadIdx.x == 0) out[blockIdx.x] = s;
+}
+
+// launch both kernels: the moments of rho (dense, device memory) into Q (device); scratch holds 2 kMomBlocks nq doubles
+template <int LMAX>
+cudaError_t launch_moments(const void* rho, int dtype, int nx, int ny, int nz, double h, const double* o, const YlmNorm& N,
+                           double* scratch, double* Q, cudaStream_t st) {
+    constexpr int NQ = (LMAX + 1) * (LMAX + 1);
+    MomArgs P;
+    P.nx = nx, P.ny = ny, P.nz = nz;
+    const double h2 = h * h, h2e = fma(h, h, -h2);
+    P.h3[0] = h2 * h;
+    P.h3[1] = fma(h2, h, -P.h3[0]) + h2e * h;
+    P.centred = 1;
+    const int ext[3] = {nx, ny, nz};
+    for (int a = 0; a < 3; ++a) {  // 2 (o + n h / 2) / h, product, sum and quotient each with its rounding error
+        const double hn = 0.5 * ext[a], p = hn * h, pe = fma(hn, h, -p);
+        const double t = p + o[a], v = t - p, te = ((p - (t - v)) + (o[a] - v)) + pe;
+        const double q = 2.0 * t / h;
+        P.off[a][0] = q;
+        P.off[a][1] = (fma(-q, h, 2.0 * t) + 2.0 * te) / h;
+        if (P.off[a][0] != 0.0 || P.off[a][1] != 0.0) P.centred = 0;
+    }
+    P.hl[0][0] = 1.0, P.hl[0][1] = 0.0;
+    for (int l = 1; l <= kMaxL; ++l) {
+        const double x = 0.25 * h, p = P.hl[l - 1][0] * x;
+        P.hl[l][0] = p;
+        P.hl[l][1] = fma(P.hl[l - 1][0], x, -p) + P.hl[l - 1][1] * x;
+    }
+    const int per16 = dtype == HG_DT_F64 ? 2 : 4;
+    const bool vec = nx % per16 == 0 && (uintptr_t)rho % 16 == 0;
+    const int th = 32 * kMomWarps;
+    if (dtype == HG_DT_F64)
+        k_moments<double, LMAX><<<kMomBlocks, th, 0, st>>>((const double*)rho, vec, P, N, scratch);
+    else
+        k_moments<float, LMAX><<<kMomBlocks, th, 0, st>>>((const float*)rho, vec, P, N, scratch);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_finish_moments<<<NQ, 32, 0, st>>>(scratch, NQ, Q);
+    return cudaGetLastError();
+}
+
+}  // namespace hg
