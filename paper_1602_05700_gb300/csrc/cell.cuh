@@ -260,8 +260,33 @@ __device__ __forceinline__ void robin_update_f32k(float a, float b, float hg, fl
     lo_o = __fsub_rn(t, __fsub_rn(hi_o, s));
 }
 
-// a double as a float and the code of its rounding remainder, and back
+// a float as the double of the same value, without the FP64 unit's conversion (normal values and zeros by shifts)
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x);
+    const unsigned ex = (u >> 23) & 0xffu;
+    if (ex == 0xffu || (ex == 0u && (u << 1) != 0u)) return (double)x;
+    const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// a double as a float and the code of its rounding remainder, and back.  For 2^-70 <= |v| < 2^127 the rounding to
+// nearest-even and the remainder (an integer of at most 29 bits in units of the double's last place, rounded once to a
+// float) come from integer instructions: the bits of the FP64 conversions and subtraction that serve the other values.
 __device__ __forceinline__ void split_f32(double v, float& hi, lo_t& lo) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+    const int ex = (int)((u >> 52) & 0x7ffu) - 1023;
+    if (ex >= -70 && ex < 127) {
+        const unsigned low = (unsigned)u & 0x1fffffffu;                            // the 29 bits a float drops
+        const unsigned top = (unsigned)(u >> 29) & 0x7fffffu;                      // the 23 it keeps
+        const bool up = low > 0x10000000u || (low == 0x10000000u && (top & 1u));
+        const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+        hi = __uint_as_float((sign | ((unsigned)(ex + 127) << 23)) + top + (up ? 1u : 0u));
+        const int r = up ? (int)low - 0x20000000 : (int)low;
+        const float unit = __uint_as_float(sign | (unsigned)(ex - 52 + 127) << 23);  // the double's last place, signed
+        lo = lo_encode(hi, __fmul_rn(__int2float_rn(r), unit));
+        return;
+    }
     hi = __double2float_rn(v);
     // a subnormal (or zero) hi keeps no compensation: its remainder is below 2^-149 and has no code
     lo = lo_encode(hi, fabsf(hi) < 1.17549435e-38f ? 0.f : __double2float_rn(__dsub_rn(v, (double)hi)));

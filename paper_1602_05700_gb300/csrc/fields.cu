@@ -2,6 +2,9 @@
 // -grad phi (arXiv 1602.05700: the force the hydro step consumes, Sec. 2), and the FP64 diagnostics of Sec. 4
 // (Eq. error) and of the steady state (Eq. Poissoneq.).  Reductions are deterministic: fixed grid, per-block
 // partial sums, one finishing block.
+#include <initializer_list>
+#include <type_traits>
+
 #include "cell.cuh"
 #include "hg_internal.cuh"
 
@@ -14,9 +17,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kPackBlocks = 1216;  // 8 per SM; one partial sum each (fits the reduction scratch)
 
-__device__ __forceinline__ double ld(const void* p, int dtype, long long i) {
-    return dtype == HG_DT_F64 ? ((const double*)p)[i] : (double)((const float*)p)[i];
-}
 __device__ __forceinline__ void st(void* p, int dtype, long long i, double v) {
     if (dtype == HG_DT_F64)
         ((double*)p)[i] = v;
@@ -41,11 +41,55 @@ __device__ __forceinline__ void for_cells(const Layout& L, F&& f) {
     }
 }
 
+// Flat numbering of the groups of W consecutive cells of a row (row j, plane k): all threads busy whatever nx is, and
+// neighbouring threads on neighbouring groups.  W is 16 bytes of the dense array where its rows allow such accesses
+// (dense_width), else 1 (coalesced single elements: groups of 4 with element stores touch every sector four times).
+// I is 32 bits wide unless the grid needs more.
+template <typename I>
+struct Group {
+    int i0, j, k;
+    long long dense;  // index of its first cell in a dense array
+};
+template <int W, typename I>
+__device__ __forceinline__ Group<I> group_of(const Layout& L, I t, unsigned gpr) {
+    const I row = t / gpr;
+    Group<I> g;
+    g.i0 = (int)(t - row * gpr) * W;
+    const I k = row / (unsigned)L.ny;
+    g.j = (int)(row - k * (unsigned)L.ny);
+    g.k = (int)k;
+    g.dense = (long long)row * L.nx + g.i0;
+    return g;
+}
+template <int W, typename I, class F>
+__device__ __forceinline__ void for_groups(const Layout& L, F&& f) {
+    const unsigned gpr = (unsigned)(L.nx / W);  // W divides nx
+    const I total = (I)gpr * (unsigned)L.ny * (unsigned)L.nz;
+    for (I t = blockIdx.x * (I)blockDim.x + threadIdx.x; t < total; t += (I)gridDim.x * blockDim.x)
+        f(group_of<W, I>(L, t, gpr));
+}
+
+template <typename T, int W>
+struct alignas(sizeof(T) * W <= 16 ? sizeof(T) * W : 16) Vec {
+    T v[W];
+};
+template <typename T, int W>
+__device__ __forceinline__ Vec<T, W> ldv(const T* p) {
+    return *reinterpret_cast<const Vec<T, W>*>(p);
+}
+template <typename T, int W>
+__device__ __forceinline__ void stv(T* p, const Vec<T, W>& x) {
+    *reinterpret_cast<Vec<T, W>*>(p) = x;
+}
+
 // Source preparation: dst = scale * (src - shift) in the grid's layout and element type, where scale =
-// (c dt)^2 4 pi G and shift = mean(rho) for periodic boundaries (else 0).  Float input to a float grid is scaled in
-// float (one rounding more than FP64, 6e-8 relative, and no slow FP64 instructions); every other combination in
-// FP64.  With SUM the same pass also accumulates sum(src) for the FP64 mass: each thread in compensated float
-// (TwoSum) or double, blocks in double, written as one partial per block (deterministic order).
+// (c dt)^2 4 pi G and shift = mean(rho) for periodic boundaries (MEAN; else nothing is subtracted).  Float input to a
+// float grid is scaled in float (one rounding more than FP64, 6e-8 relative, and no slow FP64 instructions); every other
+// combination in FP64, two operations per cell with the sum, which is what bounds it (256^3: 54 us of FP64 work; a
+// subtraction of zero and a second look at the row made it 120).  With SUM the same pass also accumulates sum(src) for
+// the FP64 mass: each thread in compensated float (TwoSum) or double, blocks in double, written as one partial per
+// block (deterministic order).  The mean is one double in memory (written by the finishing kernel of the sum pass):
+// dividing in every thread was 40 of the 46 us at 128^3.
 __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x) {
     const float t = s + x;
     const float bp = t - s;
@@ -53,57 +97,32 @@ __device__ __forceinline__ void two_sum_acc(float& s, float& c, float x) {
     s = t;
 }
 
-template <typename TS, typename TD, bool SUM>
+template <typename TS, typename TD, bool SUM, bool MEAN, int W, typename I>
 __global__ void __launch_bounds__(kThreads) k_pack(const TS* __restrict__ src, TD* __restrict__ dst, Layout L,
-                                                   const double* __restrict__ sum, double count, double scale,
-                                                   double* partial) {
+                                                   const double* __restrict__ mean, double scale, double* partial) {
     float fs = 0.f, fc = 0.f;  // compensated float accumulator (float input)
     double ds = 0.0;           // double accumulator (double input)
-    const double shift = sum ? *sum / count : 0.0;  // rho_bar = sum(rho) / cells, read on the device (no host sync)
+    constexpr bool in_float = sizeof(TS) == 4 && sizeof(TD) == 4;
+    const double shift = MEAN ? *mean : 0.0;
     const float scale32 = (float)scale, shift32 = (float)shift;
-    if constexpr (sizeof(TS) == 4 && sizeof(TD) == 4) {
-        if ((L.nx & 3) == 0 && ((uintptr_t)src & 15) == 0) {  // 16-byte groups on both sides
-            // a block takes rpb rows at a time (all its threads busy when a row has fewer groups than threads)
-            const long long rows = (long long)L.ny * L.nz;
-            const int gpr = L.nx >> 2, rpb = gpr >= (int)blockDim.x ? 1 : (int)blockDim.x / gpr;
-            const int sub = rpb == 1 ? 0 : (int)threadIdx.x / gpr, i0 = rpb == 1 ? (int)threadIdx.x : (int)threadIdx.x % gpr;
-            const int istep = rpb == 1 ? (int)blockDim.x : gpr;
-            for (long long row = (long long)blockIdx.x * rpb + sub; row < rows; row += (long long)gridDim.x * rpb) {
-                if (sub >= rpb) break;  // threads beyond rpb * gpr
-                const int j = (int)(row % L.ny), k = (int)(row / L.ny);
-                const float4* s4 = reinterpret_cast<const float4*>(src + row * L.nx);
-                float4* d4 = reinterpret_cast<float4*>(dst + L.at(0, j, k));
-                for (int i = i0; i < gpr; i += istep) {
-                    const float4 x = __ldg(s4 + i);
-                    d4[i] = make_float4(scale32 * (x.x - shift32), scale32 * (x.y - shift32), scale32 * (x.z - shift32),
-                                        scale32 * (x.w - shift32));
-                    if constexpr (SUM) {
-                        two_sum_acc(fs, fc, x.x);
-                        two_sum_acc(fs, fc, x.y);
-                        two_sum_acc(fs, fc, x.z);
-                        two_sum_acc(fs, fc, x.w);
-                    }
-                }
-            }
-        } else {
-            for_cells(L, [&](int i, int j, int k, long long c) {
-                const float x = src[c];
-                dst[L.at(i, j, k)] = scale32 * (x - shift32);
-                if constexpr (SUM) two_sum_acc(fs, fc, x);
-            });
-        }
-    } else {
-        for_cells(L, [&](int i, int j, int k, long long c) {
-            const TS x = src[c];
-            dst[L.at(i, j, k)] = (TD)(scale * ((double)x - shift));
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const Vec<TS, W> x = ldv<TS, W>(src + g.dense);
+        Vec<TD, W> y;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            if constexpr (in_float)
+                y.v[e] = scale32 * (MEAN ? x.v[e] - shift32 : x.v[e]);
+            else
+                y.v[e] = (TD)(scale * (MEAN ? (double)x.v[e] - shift : (double)x.v[e]));
             if constexpr (SUM) {
                 if constexpr (sizeof(TS) == 4)
-                    two_sum_acc(fs, fc, x);
+                    two_sum_acc(fs, fc, x.v[e]);
                 else
-                    ds += x;
+                    ds += x.v[e];
             }
-        });
-    }
+        }
+        stv<TD, W>(dst + L.at(g.i0, g.j, g.k), y);
+    });
     if constexpr (SUM) {
         __shared__ double sh[32];
         const double v = block_sum(sizeof(TS) == 4 ? (double)fs + (double)fc : ds, sh);
@@ -111,8 +130,32 @@ __global__ void __launch_bounds__(kThreads) k_pack(const TS* __restrict__ src, T
     }
 }
 
-__global__ void k_unpack(int prec, const void* p, const void* lo, void* dst, int ddt, Layout L) {
-    for_cells(L, [&](int i, int j, int k, long long c) { st(dst, ddt, c, phi_at(prec, p, lo, L.at(i, j, k))); });
+// phi^n (interior) into a dense array.  A float result is the float nearest hi + lo, one float addition; a double one
+// adds the two widened by integer instructions (widen, cell.cuh), one FP64 operation.  Through FP64 conversions this
+// kernel took 963 us at 512^3.
+template <typename TO, bool F64, int W, typename I>
+__global__ void __launch_bounds__(kThreads) k_unpack(const void* p, const void* lo, TO* __restrict__ dst, Layout L) {
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const long long q = L.at(g.i0, g.j, g.k);
+        Vec<TO, W> o;
+        if constexpr (F64) {
+            const Vec<double, W> x = ldv<double, W>((const double*)p + q);
+#pragma unroll
+            for (int e = 0; e < W; ++e) o.v[e] = (TO)x.v[e];
+        } else {
+            const Vec<float, W> h = ldv<float, W>((const float*)p + q);
+            const Vec<lo_code, W> c = ldv<lo_code, W>((const lo_code*)lo + q);
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const float l = lo_decode(h.v[e], __ushort_as_half(c.v[e]));
+                if constexpr (sizeof(TO) == 4)
+                    o.v[e] = __fadd_rn(h.v[e], l);
+                else
+                    o.v[e] = __dadd_rn(widen(h.v[e]), widen(l));
+            }
+        }
+        stv<TO, W>(dst + g.dense, o);
+    });
 }
 
 __global__ void k_unpack_ghosted(int prec, const void* p, const void* lo, double* dst, Layout L) {
@@ -129,26 +172,54 @@ __global__ void k_unpack_ghosted(int prec, const void* p, const void* lo, double
 }
 
 // seed: level n from phi, level n-1 from prev (F64 into the two buffers; F32K: hi/lo split of phi and
-// dlt = phi - prev rounded once)
-__global__ void k_seed(int prec, const void* phi, const void* prev, int sdt, void* p_cur, void* l_cur, void* p_oth,
-                       void* l_oth, void* dlt, Layout L) {
-    for_cells(L, [&](int i, int j, int k, long long c) {
-        const long long q = L.at(i, j, k);
-        const double a = ld(phi, sdt, c);
-        const double b = prev ? ld(prev, sdt, c) : a;
-        if (prec == HG_PREC_F64) {
-            ((double*)p_cur)[q] = a;
-            ((double*)p_oth)[q] = b;
+// dlt = phi - prev rounded once).  Without prev the two levels are equal, so one split serves both; the split runs in
+// integer instructions (split_f32): 375 us at 280^3 before, when each level took an FP64 subtraction and four conversions.
+template <typename TS, bool F64, int W, typename I>
+__global__ void __launch_bounds__(kThreads) k_seed(const TS* __restrict__ phi, const TS* __restrict__ prev, void* p_cur,
+                                                   void* l_cur, void* p_oth, void* l_oth, void* dlt, Layout L) {
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const long long q = L.at(g.i0, g.j, g.k);
+        const Vec<TS, W> a = ldv<TS, W>(phi + g.dense);
+        const Vec<TS, W> b = prev ? ldv<TS, W>(prev + g.dense) : a;
+        if constexpr (F64) {
+            Vec<double, W> x, y;
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                x.v[e] = (double)a.v[e];
+                y.v[e] = (double)b.v[e];
+            }
+            stv<double, W>((double*)p_cur + q, x);
+            stv<double, W>((double*)p_oth + q, y);
         } else {
-            float ha, hb;
-            lo_t la, lb;
-            split_f32(a, ha, la);
-            split_f32(b, hb, lb);
-            ((float*)p_cur)[q] = ha;
-            ((lo_t*)l_cur)[q] = la;
-            ((float*)p_oth)[q] = hb;
-            ((lo_t*)l_oth)[q] = lb;
-            ((float*)dlt)[q] = (float)(a - b);
+            Vec<float, W> ha, hb, d;
+            Vec<lo_code, W> la, lb;
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                lo_t l;
+                if constexpr (sizeof(TS) == 4) {  // a float is its own split
+                    ha.v[e] = a.v[e];
+                    la.v[e] = 0;
+                    hb.v[e] = b.v[e];
+                    lb.v[e] = 0;
+                    d.v[e] = __fsub_rn(a.v[e], b.v[e]);
+                } else {
+                    split_f32(a.v[e], ha.v[e], l);
+                    la.v[e] = __half_as_ushort(l);
+                    hb.v[e] = ha.v[e];
+                    lb.v[e] = la.v[e];
+                    d.v[e] = 0.f;
+                    if (prev) {
+                        split_f32(b.v[e], hb.v[e], l);
+                        lb.v[e] = __half_as_ushort(l);
+                        d.v[e] = (float)(a.v[e] - b.v[e]);
+                    }
+                }
+            }
+            stv<float, W>((float*)p_cur + q, ha);
+            stv<lo_code, W>((lo_code*)l_cur + q, la);
+            stv<float, W>((float*)p_oth + q, hb);
+            stv<lo_code, W>((lo_code*)l_oth + q, lb);
+            stv<float, W>((float*)dlt + q, d);
         }
     });
 }
@@ -175,21 +246,50 @@ __global__ void k_accel(int prec, const void* p, const void* lo, void* ax, void*
     });
 }
 
+// -grad phi of an FP64 grid in FP64: groups of W cells, each with its six neighbours (rows and planes out of L1 / L2),
+// six FP64 operations per cell (the sign rides on the factor: (a - b)(-s) has the bits of -(a - b) s).  256^3: 162 us of
+// FP64 work.
+template <int W, typename I>
+__global__ void __launch_bounds__(kThreads) k_accel_f64(const double* __restrict__ phi, double* __restrict__ ax,
+                                                        double* __restrict__ ay, double* __restrict__ az, Layout L,
+                                                        double inv2h) {
+    const double s = -inv2h;
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const double* p = phi + L.at(g.i0, g.j, g.k);
+        const Vec<double, W> c = ldv<double, W>(p), ys = ldv<double, W>(p - L.pitch), yn = ldv<double, W>(p + L.pitch),
+                             zm = ldv<double, W>(p - L.plane), zp = ldv<double, W>(p + L.plane);
+        const double xl = p[-1], xr = p[W];
+        Vec<double, W> x, y, z;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            x.v[e] = ((e == W - 1 ? xr : c.v[(e + 1) % W]) - (e == 0 ? xl : c.v[(e + W - 1) % W])) * s;
+            y.v[e] = (yn.v[e] - ys.v[e]) * s;
+            z.v[e] = (zp.v[e] - zm.v[e]) * s;
+        }
+        stv<double, W>(ax + g.dense, x);
+        stv<double, W>(ay + g.dense, y);
+        stv<double, W>(az + g.dense, z);
+    });
+}
+
 // Vectorised -grad phi for compensated float grids with float output (the per-hydro-step call): the work mapping
 // of the sub-step kernel (a warp per 128-cell x-row, float4 per lane, x neighbours by shuffles, a z register queue)
 // and the same arithmetic as k_accel.  HBM bytes per cell: read hi 4, lo 2; write ax, ay, az 12 = 18 B.  The kernel
 // waits on its loads (no data reuse hides them), so four blocks per SM (64 registers) beat three (71 registers):
-// 0.432 against 0.458 ms at 512^3.
+// 0.432 against 0.458 ms at 512^3.  Where the dense rows do not start on 16 bytes (nx not a multiple of 4) a lane's four
+// results cannot be stored as one word, and element stores 16 bytes apart write every sector four times: the warp's row
+// goes through shared memory instead and is stored 32 consecutive elements at a time.
 constexpr int kAccWY = 8;
 __global__ void __launch_bounds__(32 * kAccWY, 4) k_accel_f32k(const float* __restrict__ hi, const lo_t* __restrict__ lo,
                                                             float* __restrict__ ax, float* __restrict__ ay,
                                                             float* __restrict__ az, Layout L, float s, int zb) {
+    __shared__ __align__(16) float row[kAccWY][128];
     const int lane = threadIdx.x;
     const int j = blockIdx.y * kAccWY + threadIdx.y;
     if (j >= L.ny) return;
     const int i0 = blockIdx.x * 128 + lane * 4;
     const bool active = i0 < L.nx, halo = i0 <= L.nx;
-    const bool vec = (L.nx & 3) == 0 && i0 + 3 < L.nx;
+    const bool vec = (L.nx & 3) == 0;
     const int k0 = blockIdx.z * zb, k1 = min(L.nz, k0 + zb);
     auto ld4 = [](const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); };
     auto ldl4 = [](const lo_t* p) { return __ldg(reinterpret_cast<const uint2*>(p)); };
@@ -233,34 +333,35 @@ __global__ void __launch_bounds__(32 * kAccWY, 4) k_accel_f32k(const float* __re
             hr = shr;
             lr = slr;
         }
-        if (active) {
-            const float xh[6] = {hl, hc.x, hc.y, hc.z, hc.w, hr}, xl[6] = {ll, lc.x, lc.y, lc.z, lc.w, lr};
-            const float hs_[4] = {hs.x, hs.y, hs.z, hs.w}, hn_[4] = {hn.x, hn.y, hn.z, hn.w};
-            const float ls_[4] = {ls.x, ls.y, ls.z, ls.w}, ln_[4] = {ln.x, ln.y, ln.z, ln.w};
-            const float hm_[4] = {hm.x, hm.y, hm.z, hm.w}, hp_[4] = {hp.x, hp.y, hp.z, hp.w};
-            const float lm_[4] = {lm.x, lm.y, lm.z, lm.w}, lp_[4] = {lp.x, lp.y, lp.z, lp.w};
-            float ox[4], oy[4], oz[4];
+        const float xh[6] = {hl, hc.x, hc.y, hc.z, hc.w, hr}, xl[6] = {ll, lc.x, lc.y, lc.z, lc.w, lr};
+        const float hs_[4] = {hs.x, hs.y, hs.z, hs.w}, hn_[4] = {hn.x, hn.y, hn.z, hn.w};
+        const float ls_[4] = {ls.x, ls.y, ls.z, ls.w}, ln_[4] = {ln.x, ln.y, ln.z, ln.w};
+        const float hm_[4] = {hm.x, hm.y, hm.z, hm.w}, hp_[4] = {hp.x, hp.y, hp.z, hp.w};
+        const float lm_[4] = {lm.x, lm.y, lm.z, lm.w}, lp_[4] = {lp.x, lp.y, lp.z, lp.w};
+        float ox[4], oy[4], oz[4];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                ox[e] = -((xh[e + 2] - xh[e]) + (xl[e + 2] - xl[e])) * s;
-                oy[e] = -((hn_[e] - hs_[e]) + (ln_[e] - ls_[e])) * s;
-                oz[e] = -((hp_[e] - hm_[e]) + (lp_[e] - lm_[e])) * s;
-            }
-            const long long c = ((long long)k * L.ny + j) * L.nx + i0;
-            if (vec) {
-                *reinterpret_cast<float4*>(ax + c) = make_float4(ox[0], ox[1], ox[2], ox[3]);
-                *reinterpret_cast<float4*>(ay + c) = make_float4(oy[0], oy[1], oy[2], oy[3]);
-                *reinterpret_cast<float4*>(az + c) = make_float4(oz[0], oz[1], oz[2], oz[3]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (i0 + e < L.nx) {
-                        ax[c + e] = ox[e];
-                        ay[c + e] = oy[e];
-                        az[c + e] = oz[e];
-                    }
-            }
+        for (int e = 0; e < 4; ++e) {
+            ox[e] = -((xh[e + 2] - xh[e]) + (xl[e + 2] - xl[e])) * s;
+            oy[e] = -((hn_[e] - hs_[e]) + (ln_[e] - ls_[e])) * s;
+            oz[e] = -((hp_[e] - hm_[e]) + (lp_[e] - lm_[e])) * s;
         }
+        const long long c = ((long long)k * L.ny + j) * L.nx + i0;
+        auto store = [&](float* out, const float (&o)[4]) {
+            if (vec) {
+                if (active) *reinterpret_cast<float4*>(out + c) = make_float4(o[0], o[1], o[2], o[3]);
+                return;
+            }
+            float* r = row[threadIdx.y];
+            *reinterpret_cast<float4*>(r + 4 * lane) = make_float4(o[0], o[1], o[2], o[3]);
+            __syncwarp();
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (i0 - 3 * lane + 32 * e < L.nx) out[c - 3 * lane + 32 * e] = r[lane + 32 * e];
+            __syncwarp();
+        };
+        store(ax, ox);
+        store(ay, oy);
+        store(az, oz);
         hm = hc;
         hc = hp;
         lm = lc;
@@ -362,8 +463,10 @@ __global__ void __launch_bounds__(kThreads) k_sum(const void* src, int dt, long 
 }
 
 // finish: out[s] = sum (or max, per bit of maxmask) over blocks of partial[b*ns + s], fixed order
+// (with `mean`: *mean = out[0] / count)
 __global__ void __launch_bounds__(kThreads) k_finish_mixed(const double* partial, int nblocks, int ns,
-                                                           unsigned maxmask, double* out) {
+                                                           unsigned maxmask, double* out, double* mean = nullptr,
+                                                           double count = 1.0) {
     __shared__ double sh[32];
     for (int s = 0; s < ns; ++s) {
         const bool is_max = (maxmask >> s) & 1u;
@@ -374,6 +477,7 @@ __global__ void __launch_bounds__(kThreads) k_finish_mixed(const double* partial
         }
         v = block_reduce(v, sh, is_max);
         if (threadIdx.x == 0) out[s] = v;
+        if (mean && threadIdx.x == 0) *mean = v / count;
     }
 }
 
@@ -385,22 +489,56 @@ inline unsigned cells_blocks(const hg_grid* g) {
 
 }  // namespace
 
-template <bool SUM>
-static int launch_pack(hg_grid* g, const void* src, int dtype, const double* sum, double scale) {
-    const unsigned blocks = SUM ? (unsigned)kPackBlocks : cells_blocks(g);
-    const double count = (double)g->nx * g->ny * g->nz;
+// elements per 16-byte word of a dense array of type T if its rows hold whole words on 16-byte boundaries, else 1
+template <typename T>
+static int dense_width(const hg_grid* g, std::initializer_list<const void*> ptrs) {
+    constexpr int W = 16 / sizeof(T);
+    uintptr_t bits = 0;
+    for (const void* p : ptrs) bits |= (uintptr_t)p;
+    return g->nx % W == 0 && bits % 16 == 0 ? W : 1;
+}
+// groups of `w` cells are numbered in 32 bits (with room for the grid stride's overshoot)
+static bool fits32(const hg_grid* g) { return (long long)g->nx * g->ny * g->nz < (1LL << 31); }
+static unsigned group_blocks(const hg_grid* g, int w) {
+    const long long n = ((long long)g->nx * g->ny * g->nz / w + kThreads - 1) / kThreads;
+    return (unsigned)(n < (1LL << 22) ? n : 1LL << 22);
+}
+// call f with the group width (1 or the word's elements) and the index type as compile-time values
+template <typename T, class F>
+static void dispatch_groups(const hg_grid* g, int w, F&& f) {
+    constexpr int W = 16 / sizeof(T);
+    using One = std::integral_constant<int, 1>;
+    using Word = std::integral_constant<int, W>;
+    if (fits32(g)) {
+        if (w == W) f(Word(), 0u);
+        else f(One(), 0u);
+    } else {
+        if (w == W) f(Word(), 0ull);
+        else f(One(), 0ull);
+    }
+}
+
+template <typename TS, typename TD, bool SUM, bool MEAN>
+static void pack_launch(hg_grid* g, const void* src) {
+    // the narrower of the two types sets the group: 16 bytes of it
+    using T = std::conditional_t<(sizeof(TS) < sizeof(TD)), TD, TS>;
+    dispatch_groups<T>(g, dense_width<T>(g, {src}), [&](auto W, auto I) {
+        const unsigned blocks = SUM ? (unsigned)kPackBlocks : group_blocks(g, W);
+        k_pack<TS, TD, SUM, MEAN, W.value, decltype(I)><<<blocks, kThreads, 0, g->stream>>>(
+            (const TS*)src, (TD*)g->rho, g->L, g->dmean, g->src, g->red);
+    });
+}
+
+template <bool SUM, bool MEAN>
+static int launch_pack(hg_grid* g, const void* src, int dtype) {
     if (dtype == HG_DT_F32 && g->prec == HG_PREC_F32K)
-        k_pack<float, float, SUM><<<blocks, kThreads, 0, g->stream>>>((const float*)src, (float*)g->rho, g->L, sum,
-                                                                      count, scale, g->red);
+        pack_launch<float, float, SUM, MEAN>(g, src);
     else if (dtype == HG_DT_F32)
-        k_pack<float, double, SUM><<<blocks, kThreads, 0, g->stream>>>((const float*)src, (double*)g->rho, g->L, sum,
-                                                                       count, scale, g->red);
+        pack_launch<float, double, SUM, MEAN>(g, src);
     else if (g->prec == HG_PREC_F32K)
-        k_pack<double, float, SUM><<<blocks, kThreads, 0, g->stream>>>((const double*)src, (float*)g->rho, g->L, sum,
-                                                                       count, scale, g->red);
+        pack_launch<double, float, SUM, MEAN>(g, src);
     else
-        k_pack<double, double, SUM><<<blocks, kThreads, 0, g->stream>>>((const double*)src, (double*)g->rho, g->L,
-                                                                        sum, count, scale, g->red);
+        pack_launch<double, double, SUM, MEAN>(g, src);
     HG_LAUNCHED("source preparation kernel");
     return HG_OK;
 }
@@ -413,9 +551,9 @@ int prepare_source(hg_grid* g, const void* src, int dtype) {
     g->mass_pending = 1;
     if (g->bc == HG_BC_PERIODIC) {
         if ((rc = reduce_sum(g, src, dtype, g->dsum))) return rc;
-        return launch_pack<false>(g, src, dtype, g->dsum, g->src);
+        return launch_pack<false, true>(g, src, dtype);
     }
-    if ((rc = launch_pack<true>(g, src, dtype, nullptr, g->src))) return rc;
+    if ((rc = launch_pack<true, false>(g, src, dtype))) return rc;
     k_finish_mixed<<<1, kThreads, 0, g->stream>>>(g->red, kPackBlocks, 1, 0u, g->dsum);
     HG_LAUNCHED("sum finish kernel");
     return HG_OK;
@@ -434,7 +572,19 @@ int sync_mass(hg_grid* g) {
 }
 
 int unpack_phi(hg_grid* g, void* dst, int dtype) {
-    k_unpack<<<cells_blocks(g), kThreads, 0, g->stream>>>(g->prec, g->phi[g->cur], g->lo[g->cur], dst, dtype, g->L);
+    const void *p = g->phi[g->cur], *lo = g->lo[g->cur];
+    auto run = [&](auto out, auto f64) {
+        using TO = decltype(out);
+        dispatch_groups<TO>(g, dense_width<TO>(g, {dst}), [&](auto W, auto I) {
+            k_unpack<TO, f64.value, W.value, decltype(I)>
+                <<<group_blocks(g, W), kThreads, 0, g->stream>>>(p, lo, (TO*)dst, g->L);
+        });
+    };
+    const bool f64 = g->prec == HG_PREC_F64;
+    if (dtype == HG_DT_F64)
+        f64 ? run(0.0, std::true_type()) : run(0.0, std::false_type());
+    else
+        f64 ? run(0.f, std::true_type()) : run(0.f, std::false_type());
     HG_LAUNCHED("unpack kernel");
     return HG_OK;
 }
@@ -447,8 +597,19 @@ int unpack_phi_ghosted(hg_grid* g, double* dst) {
 
 int set_phi_device(hg_grid* g, const void* phi, const void* prev, int dtype) {
     int oth = 1 - g->cur;
-    k_seed<<<cells_blocks(g), kThreads, 0, g->stream>>>(g->prec, phi, prev, dtype, g->phi[g->cur], g->lo[g->cur],
-                                                        g->phi[oth], g->lo[oth], g->dlt[g->dcur], g->L);
+    auto run = [&](auto in, auto f64) {
+        using TS = decltype(in);
+        dispatch_groups<TS>(g, dense_width<TS>(g, {phi, prev}), [&](auto W, auto I) {
+            k_seed<TS, f64.value, W.value, decltype(I)><<<group_blocks(g, W), kThreads, 0, g->stream>>>(
+                (const TS*)phi, (const TS*)prev, g->phi[g->cur], g->lo[g->cur], g->phi[oth], g->lo[oth],
+                g->dlt[g->dcur], g->L);
+        });
+    };
+    const bool f64 = g->prec == HG_PREC_F64;
+    if (dtype == HG_DT_F64)
+        f64 ? run(0.0, std::true_type()) : run(0.0, std::false_type());
+    else
+        f64 ? run(0.f, std::true_type()) : run(0.f, std::false_type());
     HG_LAUNCHED("seed kernel");
     return HG_OK;
 }
@@ -462,6 +623,11 @@ int accel(hg_grid* g, void* ax, void* ay, void* az, int dtype) {
         k_accel_f32k<<<grid, block, 0, g->stream>>>((const float*)g->phi[g->cur], (const lo_t*)g->lo[g->cur],
                                                     (float*)ax, (float*)ay, (float*)az, g->L,
                                                     (float)(1.0 / (2.0 * g->h)), zb);
+    } else if (g->prec == HG_PREC_F64 && dtype == HG_DT_F64) {
+        dispatch_groups<double>(g, dense_width<double>(g, {ax, ay, az}), [&](auto W, auto I) {
+            k_accel_f64<W.value, decltype(I)><<<group_blocks(g, W), kThreads, 0, g->stream>>>(
+                (const double*)g->phi[g->cur], (double*)ax, (double*)ay, (double*)az, g->L, 1.0 / (2.0 * g->h));
+        });
     } else {
         k_accel<<<cells_blocks(g), kThreads, 0, g->stream>>>(g->prec, g->phi[g->cur], g->lo[g->cur], ax, ay, az,
                                                              dtype, g->L, 1.0 / (2.0 * g->h));
@@ -513,7 +679,7 @@ int reduce_sum(hg_grid* g, const void* dense, int dtype, double* out_dev) {
     long long n = (long long)g->nx * g->ny * g->nz;
     k_sum<<<kPackBlocks, kThreads, 0, g->stream>>>(dense, dtype, n, g->red);
     HG_LAUNCHED("sum kernel");
-    k_finish_mixed<<<1, kThreads, 0, g->stream>>>(g->red, kPackBlocks, 1, 0u, out_dev);
+    k_finish_mixed<<<1, kThreads, 0, g->stream>>>(g->red, kPackBlocks, 1, 0u, out_dev, g->dmean, (double)n);
     HG_LAUNCHED("sum finish kernel");
     return HG_OK;
 }

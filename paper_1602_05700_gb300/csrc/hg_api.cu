@@ -275,11 +275,12 @@ static int init_grid(hg_grid** out, int nx, int ny, int nz, double h, const doub
     if (rc == HG_OK) {
         g->red_elems = reduction_scratch_elems();
         e = cudaMalloc(&g->red, (size_t)g->red_elems * sizeof(double));
-        if (e == cudaSuccess) e = cudaMalloc(&g->dres, (kMaxQ + 2) * sizeof(double));
-        if (e == cudaSuccess) e = cudaMemsetAsync(g->dres, 0, (kMaxQ + 2) * sizeof(double), g->stream);
+        if (e == cudaSuccess) e = cudaMalloc(&g->dres, (kMaxQ + 3) * sizeof(double));
+        if (e == cudaSuccess) e = cudaMemsetAsync(g->dres, 0, (kMaxQ + 3) * sizeof(double), g->stream);
         if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(reduction scratch)");
         g->dsum = g->dres + kMaxQ;
         g->derr = (int*)(g->dres + kMaxQ + 1);
+        g->dmean = g->dres + kMaxQ + 2;
     }
     if (rc == HG_OK) {
         e = cudaStreamSynchronize(g->stream);

@@ -159,6 +159,7 @@ struct hg_grid {
     long long red_elems;
     double* dres;   // small device result buffer
     double* dsum;   // sum(rho) of the last density, written on the device by the source preparation
+    double* dmean;  // its mean (periodic boundaries), likewise
     int* derr;      // device error word: value 1 a bounded wait in a kernel gave up (HG_ERR_TIMEOUT), value 2 a debug
                     // index check failed (HG_ERR_BOUNDS)
     int mass_pending;  // mass / rho_bar below not yet read back from dsum

@@ -56,16 +56,16 @@ template <typename T>
 __global__ void __launch_bounds__(hg::kRedThreads) k_max_speed(const T* __restrict__ U, long long n, T gamma, T gm1,
                                                               double* __restrict__ red) {
     __shared__ double sh[32];
-    double m = 0.0;
+    T big = T(0);  // the maximum in the state's precision: widening every cell's speed cost more than its square roots
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
         T u[5], w[5];
 #pragma unroll
         for (int q = 0; q < 5; ++q) u[q] = U[q * n + c];
         cons_to_prim(gm1, u, w);
         const T s = sqrt((w[1] * w[1] + w[2] * w[2]) + w[3] * w[3]) + sqrt(gamma * w[4] / w[0]);
-        if ((double)s > m) m = (double)s;
+        if (s > big) big = s;
     }
-    m = hg::block_reduce(m, sh, true);
+    const double m = hg::block_reduce((double)big, sh, true);
     if (threadIdx.x == 0) red[blockIdx.x] = m;
 }
 

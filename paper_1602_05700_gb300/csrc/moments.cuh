@@ -24,6 +24,7 @@
 // 3.2e-16 / 5.3e-15 -> 2.4e-16 / 1.6e-15.
 #pragma once
 
+#include "cell.cuh"
 #include "hg_internal.cuh"
 
 namespace hg {
@@ -100,15 +101,6 @@ __device__ __forceinline__ void dd_warp(double& s, double& e) {
     }
 }
 
-// a float as the double of the same value, without the FP64 conversion (normal values and zeros by shifts)
-__device__ __forceinline__ double widen(float x) {
-    const unsigned u = __float_as_uint(x);
-    const unsigned ex = (u >> 23) & 0xffu;
-    if (ex == 0xffu || (ex == 0u && (u << 1) != 0u)) return (double)x;
-    const unsigned hi = (u & 0x80000000u) | (ex ? ((u & 0x7fffffffu) >> 3) + 0x38000000u : 0u);
-    return __hiloint2double((int)hi, (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ bool nonzero(float x) { return (__float_as_uint(x) << 1) != 0u; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 
