@@ -15,6 +15,7 @@
 // Kernels here: add an injection into the shadow state, accumulate sum_m lambda^m (float pairs for the compensated
 // precision, double for FP64), and turn the sum into the gradient.
 #include "cell.cuh"
+#include "groups.cuh"
 #include "hg_internal.cuh"
 
 namespace hg {
@@ -23,78 +24,91 @@ namespace {
 
 constexpr int kThreads = 256;
 
-template <class F>
-__device__ __forceinline__ void for_cells(const Layout& L, F&& f) {
-    const long long rows = (long long)L.ny * L.nz;
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x) {
-        const int j = (int)(row % L.ny), k = (int)(row / L.ny);
-        const long long base = row * L.nx;
-        for (int i = threadIdx.x; i < L.nx; i += blockDim.x) f(L.at(i, j, k), base + i);
+// lambda^m += v on the interior; for the compensated state the increment dlt = lambda^m - lambda^{m+1} moves too.  A
+// double enters as the float pair nearest to it.
+template <typename T, bool F64, int W, typename I>
+__global__ void __launch_bounds__(kThreads) k_inject(const T* __restrict__ v, void* hi, void* lo, void* dlt, Layout L) {
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const long long q = L.at(g.i0, g.j, g.k);
+        const Vec<T, W> x = ldv<T, W>(v + g.dense);
+        if constexpr (F64) {
+            Vec<double, W> p = ldv<double, W>((double*)hi + q);
+#pragma unroll
+            for (int e = 0; e < W; ++e) p.v[e] += (double)x.v[e];
+            stv<double, W>((double*)hi + q, p);
+        } else {
+            Vec<float, W> h = ldv<float, W>((float*)hi + q), d = ldv<float, W>((float*)dlt + q);
+            Vec<lo_code, W> c = ldv<lo_code, W>((lo_code*)lo + q);
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const float xh = (float)x.v[e];
+                const float xl = sizeof(T) == 4 ? 0.f : (float)((double)x.v[e] - (double)xh);
+                float s, r;
+                two_sum(h.v[e], xh, s, r);
+                const float t = (lo_decode(h.v[e], __ushort_as_half(c.v[e])) + xl) + r;
+                const float hn = s + t;
+                h.v[e] = hn;
+                c.v[e] = __half_as_ushort(lo_encode(hn, t - (hn - s)));
+                d.v[e] += xh;
+            }
+            stv<float, W>((float*)hi + q, h);
+            stv<lo_code, W>((lo_code*)lo + q, c);
+            stv<float, W>((float*)dlt + q, d);
+        }
+    });
+}
+
+// acc += lambda^m on the interior, for grids whose sub-step does not do it on the way (stencil_small.cu).  All three
+// arrays are padded, so groups of 4 (rows have room for the last one) whatever nx is.
+template <bool F64>
+__global__ void __launch_bounds__(kThreads) k_accumulate(const void* hi, const void* lo, void* acc_a, void* acc_b, Layout L,
+                                                         unsigned gpr) {
+    for (long long t = blockIdx.x * (long long)kThreads + threadIdx.x; t < (long long)gpr * L.ny * L.nz;
+         t += (long long)gridDim.x * kThreads) {
+        const long long row = t / gpr;
+        const long long q = L.at((int)(t - row * gpr) * 4, (int)(row % L.ny), (int)(row / L.ny));
+        if constexpr (F64) {
+            Vec<double, 4> a = ldv<double, 4>((double*)acc_a + q);
+            const Vec<double, 4> x = ldv<double, 4>((const double*)hi + q);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a.v[e] += x.v[e];
+            stv<double, 4>((double*)acc_a + q, a);
+        } else {
+            Vec<float, 4> a = ldv<float, 4>((float*)acc_a + q), b = ldv<float, 4>((float*)acc_b + q);
+            const Vec<float, 4> h = ldv<float, 4>((const float*)hi + q);
+            const Vec<lo_code, 4> c = ldv<lo_code, 4>((const lo_code*)lo + q);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                accumulate_f32k(a.v[e], b.v[e], h.v[e], lo_decode(h.v[e], __ushort_as_half(c.v[e])));
+            stv<float, 4>((float*)acc_a + q, a);
+            stv<float, 4>((float*)acc_b + q, b);
+        }
     }
 }
 
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float bp = s - a;
-    e = (a - (s - bp)) + (b - bp);
-}
-
-// lambda^m += v on the interior; for the compensated state the increment dlt = lambda^m - lambda^{m+1} moves too
-__global__ void k_inject(int prec, const void* v, int vdt, void* hi, void* lo, void* dlt, Layout L) {
-    for_cells(L, [&](long long q, long long c) {
-        const double x = vdt == HG_DT_F64 ? ((const double*)v)[c] : (double)((const float*)v)[c];
-        if (prec == HG_PREC_F64) {
-            ((double*)hi)[q] += x;
-        } else {
-            float* h = (float*)hi;
-            lo_t* l = (lo_t*)lo;
-            const float xh = (float)x, xl = (float)(x - (double)xh);
-            const float h0 = h[q];
-            float s, e;
-            two_sum(h0, xh, s, e);
-            const float t = (lo_decode(h0, l[q]) + xl) + e;
-            const float hn = s + t;
-            h[q] = hn;
-            l[q] = lo_encode(hn, t - (hn - s));
-            ((float*)dlt)[q] += xh;
-        }
-    });
-}
-
-// acc += lambda^m on the interior
-__global__ void k_accumulate(int prec, const void* hi, const void* lo, void* acc_a, void* acc_b, Layout L) {
-    for_cells(L, [&](long long q, long long) {
-        if (prec == HG_PREC_F64) {
-            ((double*)acc_a)[q] += ((const double*)hi)[q];
-        } else {
-            float* a = (float*)acc_a;
-            float* b = (float*)acc_b;
-            float s, e;
-            const float h = ((const float*)hi)[q];
-            two_sum(a[q], h, s, e);
-            const float t = b[q] + (e + lo_decode(h, ((const lo_t*)lo)[q]));
-            a[q] = s + t;
-            b[q] = t - (a[q] - s);
-        }
-    });
-}
-
-// out = scale * acc - shift (dense, dtype); with want_sum the same pass leaves per-block partial sums of scale*acc
-__global__ void __launch_bounds__(kThreads) k_grad(int prec, const void* acc_a, const void* acc_b, void* out, int odt,
-                                                   Layout L, double scale, double shift, double* partial) {
-    __shared__ double sh[32];
+// out = scale * acc - shift (dense); with SUM the same pass leaves per-block partial sums of scale*acc
+template <typename TO, bool F64, bool SUM, int W, typename I>
+__global__ void __launch_bounds__(kThreads) k_grad(const void* acc_a, const void* acc_b, TO* __restrict__ out, Layout L,
+                                                   double scale, double shift, double* partial) {
     double sum = 0.0;
-    for_cells(L, [&](long long q, long long c) {
-        const double a = prec == HG_PREC_F64 ? ((const double*)acc_a)[q]
-                                             : (double)((const float*)acc_a)[q] + (double)((const float*)acc_b)[q];
-        const double gval = scale * a;
-        sum += gval;
-        if (odt == HG_DT_F64)
-            ((double*)out)[c] = gval - shift;
-        else
-            ((float*)out)[c] = (float)(gval - shift);
+    for_groups<W, I>(L, [&](const Group<I>& g) {
+        const long long q = L.at(g.i0, g.j, g.k);
+        Vec<TO, W> o;
+#pragma unroll
+        for (int e = 0; e < W; ++e) {
+            double a;
+            if constexpr (F64)
+                a = ((const double*)acc_a)[q + e];
+            else
+                a = __dadd_rn(widen(((const float*)acc_a)[q + e]), widen(((const float*)acc_b)[q + e]));
+            const double gval = __dmul_rn(scale, a);
+            if constexpr (SUM) sum += gval;
+            o.v[e] = (TO)(shift == 0.0 ? gval : __dsub_rn(gval, shift));
+        }
+        stv<TO, W>(out + g.dense, o);
     });
-    if (partial) {
+    if constexpr (SUM) {
+        __shared__ double sh[32];
         const double v = block_sum(sum, sh);
         if (threadIdx.x == 0) partial[blockIdx.x] = v;
     }
@@ -108,25 +122,39 @@ __global__ void k_finish_sum(const double* partial, int n, double* out) {
     if (threadIdx.x == 0) *out = v;
 }
 
-unsigned blocks_for(const Layout& L) {
-    long long rows = (long long)L.ny * L.nz;
-    return (unsigned)(rows < kRedBlocks ? rows : kRedBlocks);
+// f(dtype tag, FP64 grid?) with compile-time values
+template <class F>
+void by_type(bool f64_data, bool f64_grid, F&& f) {
+    if (f64_data)
+        f64_grid ? f(0.0, std::true_type()) : f(0.0, std::false_type());
+    else
+        f64_grid ? f(0.f, std::true_type()) : f(0.f, std::false_type());
 }
 
 }  // namespace
 
 int adjoint_inject(hg_grid* a, const void* v, int vdt) {
     hg_grid* g = a;
-    k_inject<<<blocks_for(a->L), kThreads, 0, a->stream>>>(a->prec, v, vdt, a->phi[a->cur], a->lo[a->cur],
-                                                           a->dlt[a->dcur], a->L);
+    by_type(vdt == HG_DT_F64, a->prec == HG_PREC_F64, [&](auto in, auto f64) {
+        using T = decltype(in);
+        dispatch_groups<T>(a->L, dense_width<T>(a->L, {v}), [&](auto W, auto I) {
+            k_inject<T, f64.value, W.value, decltype(I)><<<group_blocks(a->L, W), kThreads, 0, a->stream>>>(
+                (const T*)v, a->phi[a->cur], a->lo[a->cur], a->dlt[a->dcur], a->L);
+        });
+    });
     HG_LAUNCHED("adjoint injection kernel");
     return HG_OK;
 }
 
 int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b) {
     hg_grid* g = a;
-    k_accumulate<<<blocks_for(a->L), kThreads, 0, a->stream>>>(a->prec, a->phi[a->cur], a->lo[a->cur], acc_a, acc_b,
-                                                               a->L);
+    const unsigned gpr = (unsigned)((a->nx + 3) / 4);
+    const long long n = ((long long)gpr * a->ny * a->nz + kThreads - 1) / kThreads;
+    const unsigned blocks = (unsigned)(n < (1LL << 22) ? n : 1LL << 22);
+    if (a->prec == HG_PREC_F64)
+        k_accumulate<true><<<blocks, kThreads, 0, a->stream>>>(a->phi[a->cur], nullptr, acc_a, acc_b, a->L, gpr);
+    else
+        k_accumulate<false><<<blocks, kThreads, 0, a->stream>>>(a->phi[a->cur], a->lo[a->cur], acc_a, acc_b, a->L, gpr);
     HG_LAUNCHED("adjoint accumulation kernel");
     return HG_OK;
 }
@@ -135,21 +163,30 @@ int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b) {
 int adjoint_gradient(hg_grid* a, const void* acc_a, const void* acc_b, void* out, int odt, double* scratch) {
     hg_grid* g = a;
     const double scale = -a->src;
-    const unsigned nb = blocks_for(a->L);
+    auto pass = [&](auto sum, double shift) {
+        by_type(odt == HG_DT_F64, a->prec == HG_PREC_F64, [&](auto o, auto f64) {
+            using TO = decltype(o);
+            dispatch_groups<TO>(a->L, dense_width<TO>(a->L, {out}), [&](auto W, auto I) {
+                const unsigned blocks = sum.value ? (unsigned)kRedBlocks : group_blocks(a->L, W);
+                k_grad<TO, f64.value, sum.value, W.value, decltype(I)>
+                    <<<blocks, kThreads, 0, a->stream>>>(acc_a, acc_b, (TO*)out, a->L, scale, shift, scratch);
+            });
+        });
+    };
     if (a->bc != HG_BC_PERIODIC) {
-        k_grad<<<nb, kThreads, 0, a->stream>>>(a->prec, acc_a, acc_b, out, odt, a->L, scale, 0.0, nullptr);
+        pass(std::false_type(), 0.0);
         HG_LAUNCHED("adjoint gradient kernel");
         return HG_OK;
     }
-    k_grad<<<nb, kThreads, 0, a->stream>>>(a->prec, acc_a, acc_b, out, odt, a->L, scale, 0.0, scratch);
+    pass(std::true_type(), 0.0);
     HG_LAUNCHED("adjoint gradient kernel");
-    k_finish_sum<<<1, kThreads, 0, a->stream>>>(scratch, (int)nb, scratch + kRedBlocks);
+    k_finish_sum<<<1, kThreads, 0, a->stream>>>(scratch, kRedBlocks, scratch + kRedBlocks);
     HG_LAUNCHED("adjoint gradient sum kernel");
     double sum = 0.0;
     HG_CUDA(cudaMemcpyAsync(&sum, scratch + kRedBlocks, sizeof(double), cudaMemcpyDeviceToHost, a->stream));
     HG_CUDA(cudaStreamSynchronize(a->stream));
     const double mean = sum / ((double)a->nx * a->ny * a->nz);
-    k_grad<<<nb, kThreads, 0, a->stream>>>(a->prec, acc_a, acc_b, out, odt, a->L, scale, mean, nullptr);
+    pass(std::false_type(), mean);
     HG_LAUNCHED("adjoint gradient kernel");
     return HG_OK;
 }

@@ -260,6 +260,20 @@ __device__ __forceinline__ void robin_update_f32k(float a, float b, float hg, fl
     lo_o = __fsub_rn(t, __fsub_rn(hi_o, s));
 }
 
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+    s = __fadd_rn(a, b);
+    const float bp = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bp)), __fsub_rn(b, bp));
+}
+// (a, b) += h + l: the adjoint's running sum of compensated values, a float pair
+__device__ __forceinline__ void accumulate_f32k(float& a, float& b, float h, float l) {
+    float s, e;
+    two_sum(a, h, s, e);
+    const float t = __fadd_rn(b, __fadd_rn(e, l));
+    a = __fadd_rn(s, t);
+    b = __fsub_rn(t, __fsub_rn(a, s));
+}
+
 // a float as the double of the same value, without the FP64 unit's conversion (normal values and zeros by shifts)
 __device__ __forceinline__ double widen(float x) {
     const unsigned u = __float_as_uint(x);

@@ -2,10 +2,8 @@
 // -grad phi (arXiv 1602.05700: the force the hydro step consumes, Sec. 2), and the FP64 diagnostics of Sec. 4
 // (Eq. error) and of the steady state (Eq. Poissoneq.).  Reductions are deterministic: fixed grid, per-block
 // partial sums, one finishing block.
-#include <initializer_list>
-#include <type_traits>
-
 #include "cell.cuh"
+#include "groups.cuh"
 #include "hg_internal.cuh"
 
 namespace hg {
@@ -39,47 +37,6 @@ __device__ __forceinline__ void for_cells(const Layout& L, F&& f) {
         const long long base = row * L.nx;
         for (int i = threadIdx.x; i < L.nx; i += blockDim.x) f(i, j, k, base + i);
     }
-}
-
-// Flat numbering of the groups of W consecutive cells of a row (row j, plane k): all threads busy whatever nx is, and
-// neighbouring threads on neighbouring groups.  W is 16 bytes of the dense array where its rows allow such accesses
-// (dense_width), else 1 (coalesced single elements: groups of 4 with element stores touch every sector four times).
-// I is 32 bits wide unless the grid needs more.
-template <typename I>
-struct Group {
-    int i0, j, k;
-    long long dense;  // index of its first cell in a dense array
-};
-template <int W, typename I>
-__device__ __forceinline__ Group<I> group_of(const Layout& L, I t, unsigned gpr) {
-    const I row = t / gpr;
-    Group<I> g;
-    g.i0 = (int)(t - row * gpr) * W;
-    const I k = row / (unsigned)L.ny;
-    g.j = (int)(row - k * (unsigned)L.ny);
-    g.k = (int)k;
-    g.dense = (long long)row * L.nx + g.i0;
-    return g;
-}
-template <int W, typename I, class F>
-__device__ __forceinline__ void for_groups(const Layout& L, F&& f) {
-    const unsigned gpr = (unsigned)(L.nx / W);  // W divides nx
-    const I total = (I)gpr * (unsigned)L.ny * (unsigned)L.nz;
-    for (I t = blockIdx.x * (I)blockDim.x + threadIdx.x; t < total; t += (I)gridDim.x * blockDim.x)
-        f(group_of<W, I>(L, t, gpr));
-}
-
-template <typename T, int W>
-struct alignas(sizeof(T) * W <= 16 ? sizeof(T) * W : 16) Vec {
-    T v[W];
-};
-template <typename T, int W>
-__device__ __forceinline__ Vec<T, W> ldv(const T* p) {
-    return *reinterpret_cast<const Vec<T, W>*>(p);
-}
-template <typename T, int W>
-__device__ __forceinline__ void stv(T* p, const Vec<T, W>& x) {
-    *reinterpret_cast<Vec<T, W>*>(p) = x;
 }
 
 // Source preparation: dst = scale * (src - shift) in the grid's layout and element type, where scale =
@@ -489,41 +446,12 @@ inline unsigned cells_blocks(const hg_grid* g) {
 
 }  // namespace
 
-// elements per 16-byte word of a dense array of type T if its rows hold whole words on 16-byte boundaries, else 1
-template <typename T>
-static int dense_width(const hg_grid* g, std::initializer_list<const void*> ptrs) {
-    constexpr int W = 16 / sizeof(T);
-    uintptr_t bits = 0;
-    for (const void* p : ptrs) bits |= (uintptr_t)p;
-    return g->nx % W == 0 && bits % 16 == 0 ? W : 1;
-}
-// groups of `w` cells are numbered in 32 bits (with room for the grid stride's overshoot)
-static bool fits32(const hg_grid* g) { return (long long)g->nx * g->ny * g->nz < (1LL << 31); }
-static unsigned group_blocks(const hg_grid* g, int w) {
-    const long long n = ((long long)g->nx * g->ny * g->nz / w + kThreads - 1) / kThreads;
-    return (unsigned)(n < (1LL << 22) ? n : 1LL << 22);
-}
-// call f with the group width (1 or the word's elements) and the index type as compile-time values
-template <typename T, class F>
-static void dispatch_groups(const hg_grid* g, int w, F&& f) {
-    constexpr int W = 16 / sizeof(T);
-    using One = std::integral_constant<int, 1>;
-    using Word = std::integral_constant<int, W>;
-    if (fits32(g)) {
-        if (w == W) f(Word(), 0u);
-        else f(One(), 0u);
-    } else {
-        if (w == W) f(Word(), 0ull);
-        else f(One(), 0ull);
-    }
-}
-
 template <typename TS, typename TD, bool SUM, bool MEAN>
 static void pack_launch(hg_grid* g, const void* src) {
     // the narrower of the two types sets the group: 16 bytes of it
     using T = std::conditional_t<(sizeof(TS) < sizeof(TD)), TD, TS>;
-    dispatch_groups<T>(g, dense_width<T>(g, {src}), [&](auto W, auto I) {
-        const unsigned blocks = SUM ? (unsigned)kPackBlocks : group_blocks(g, W);
+    dispatch_groups<T>(g->L, dense_width<T>(g->L, {src}), [&](auto W, auto I) {
+        const unsigned blocks = SUM ? (unsigned)kPackBlocks : group_blocks(g->L, W);
         k_pack<TS, TD, SUM, MEAN, W.value, decltype(I)><<<blocks, kThreads, 0, g->stream>>>(
             (const TS*)src, (TD*)g->rho, g->L, g->dmean, g->src, g->red);
     });
@@ -575,9 +503,9 @@ int unpack_phi(hg_grid* g, void* dst, int dtype) {
     const void *p = g->phi[g->cur], *lo = g->lo[g->cur];
     auto run = [&](auto out, auto f64) {
         using TO = decltype(out);
-        dispatch_groups<TO>(g, dense_width<TO>(g, {dst}), [&](auto W, auto I) {
+        dispatch_groups<TO>(g->L, dense_width<TO>(g->L, {dst}), [&](auto W, auto I) {
             k_unpack<TO, f64.value, W.value, decltype(I)>
-                <<<group_blocks(g, W), kThreads, 0, g->stream>>>(p, lo, (TO*)dst, g->L);
+                <<<group_blocks(g->L, W), kThreads, 0, g->stream>>>(p, lo, (TO*)dst, g->L);
         });
     };
     const bool f64 = g->prec == HG_PREC_F64;
@@ -599,8 +527,8 @@ int set_phi_device(hg_grid* g, const void* phi, const void* prev, int dtype) {
     int oth = 1 - g->cur;
     auto run = [&](auto in, auto f64) {
         using TS = decltype(in);
-        dispatch_groups<TS>(g, dense_width<TS>(g, {phi, prev}), [&](auto W, auto I) {
-            k_seed<TS, f64.value, W.value, decltype(I)><<<group_blocks(g, W), kThreads, 0, g->stream>>>(
+        dispatch_groups<TS>(g->L, dense_width<TS>(g->L, {phi, prev}), [&](auto W, auto I) {
+            k_seed<TS, f64.value, W.value, decltype(I)><<<group_blocks(g->L, W), kThreads, 0, g->stream>>>(
                 (const TS*)phi, (const TS*)prev, g->phi[g->cur], g->lo[g->cur], g->phi[oth], g->lo[oth],
                 g->dlt[g->dcur], g->L);
         });
@@ -624,8 +552,8 @@ int accel(hg_grid* g, void* ax, void* ay, void* az, int dtype) {
                                                     (float*)ax, (float*)ay, (float*)az, g->L,
                                                     (float)(1.0 / (2.0 * g->h)), zb);
     } else if (g->prec == HG_PREC_F64 && dtype == HG_DT_F64) {
-        dispatch_groups<double>(g, dense_width<double>(g, {ax, ay, az}), [&](auto W, auto I) {
-            k_accel_f64<W.value, decltype(I)><<<group_blocks(g, W), kThreads, 0, g->stream>>>(
+        dispatch_groups<double>(g->L, dense_width<double>(g->L, {ax, ay, az}), [&](auto W, auto I) {
+            k_accel_f64<W.value, decltype(I)><<<group_blocks(g->L, W), kThreads, 0, g->stream>>>(
                 (const double*)g->phi[g->cur], (double*)ax, (double*)ay, (double*)az, g->L, 1.0 / (2.0 * g->h));
         });
     } else {

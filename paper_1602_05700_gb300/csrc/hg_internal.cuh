@@ -246,7 +246,8 @@ int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cud
 
 // kernels' host launchers (each returns HG_OK or an error code)
 int launch_step_single(hg_grid* g);                  // one sub-step: cur -> 1-cur, all ghosts (stencil.cu)
-int launch_step_small(hg_grid* g);                   // the same for a small grid (stencil_small.cu)
+bool small_grid(const hg_grid* g);                   // whether launch_step_small serves this grid (stencil.cu)
+int launch_step_small(hg_grid* g, void* acc_a = nullptr, void* acc_b = nullptr);  // a small grid's (stencil_small.cu)
 int adjoint_inject(hg_grid* a, const void* v, int vdt);
 int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b);
 int adjoint_gradient(hg_grid* a, const void* acc_a, const void* acc_b, void* out, int odt, double* scratch);

@@ -233,15 +233,6 @@ __device__ __forceinline__ void sweep_f64_any(const SweepArgs& A, int bx, int by
 
 constexpr int kWY = 8;
 
-// Whether a single grid's sub-step runs as one thread per group of cells (stencil_small.cu).  The line lies where the
-// marching kernels overtake it (measured on cubes): compensated float 224^3 (60.7 against 61.2 us; 192^3 38.5 against
-// 45.6, 256^3 88 against 80), FP64 between 192^3 (107 against 131 us) and 256^3 (246 against 216).  A pinned block
-// depth (hg_set_block_depth) asks for the marching sweep.
-bool small_grid(const hg_grid* g) {
-    const long long n = (long long)g->nx * g->ny * g->nz;
-    return g->zb == 0 && n <= (g->prec == HG_PREC_F32K ? 11500000LL : 8000000LL);
-}
-
 int zchunk(const hg_grid* g) {
     // compensated-float grids (TMA-staged sweep): short chunks, many blocks -- the stage ring hides the z warm-up,
     // and fine blocks balance the SMs (measured at 512^3: 8 planes beat 16-64)
@@ -342,12 +333,21 @@ __global__ void __launch_bounds__(32 * WY, 2) k_batch_f64(const TmaEntry* __rest
 
 }  // namespace
 
-// the sweep arguments of grid g for the sub-step cur -> 1 - cur, with z chunks of zb planes (0 = default rule)
+// Whether a single grid's sub-step runs as one thread per group of cells (stencil_small.cu).  The line lies where the
+// marching kernels overtake it (measured on cubes): compensated float 224^3 (60.7 against 61.2 us; 192^3 38.5 against
+// 45.6, 256^3 88 against 80), FP64 between 192^3 (107 against 131 us) and 256^3 (246 against 216).  A pinned block
+// depth (hg_set_block_depth) asks for the marching sweep.
+bool small_grid(const hg_grid* g) {
+    const long long n = (long long)g->nx * g->ny * g->nz;
+    return g->zb == 0 && n <= (g->prec == HG_PREC_F32K ? 11500000LL : 8000000LL);
+}
+
 int f64_cells_per_lane(int nx) {
     const long long w4 = (nx + 127) / 128 * 128LL, w1 = (nx + 31) / 32 * 32LL;
     return w1 < w4 ? 1 : 4;
 }
 
+// the sweep arguments of grid g for the sub-step cur -> 1 - cur, with z chunks of zb planes (0 = default rule)
 SweepArgs sweep_args(const hg_grid* g, int zb, int cpl) {
     SweepArgs A;
     const int nxt = 1 - g->cur;

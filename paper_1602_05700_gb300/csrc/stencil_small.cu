@@ -10,6 +10,9 @@
 // copy.  One launch per sub-step, by programmatic dependent launch: its blocks are resident, with their indices
 // computed, when the previous sub-step ends.
 //
+// The adjoint's reverse sub-steps (ADJ) add level n to their running sum here, from the registers that hold it: a pass of
+// its own took 32 us at 128^3 (float) beside the 9 us of the sub-step; this variant takes 12.
+//
 // Measured (Robin, us per sub-step, marching kernel with its own ghost launches -> this one):
 //   compensated float  32^3 14.4 -> 2.5, 64^3 14.4 -> 3.7, 128^3 16.4 -> 9.0, 192^3 46.6 -> 38.5, 256^3 80.7 -> 88
 //   FP64               32^3 21.2 -> 3.9, 64^3 18.0 -> 7.9, 128^3 39.6 -> 31.4, 192^3 139 -> 107, 256^3 228 -> 246
@@ -37,7 +40,9 @@ __device__ __forceinline__ bool small_cell(const Layout& L, unsigned t, unsigned
     return k < L.nz;
 }
 
-__global__ void __launch_bounds__(kSmallThreads) k_small_f32k(const SweepArgs A, unsigned gblocks, unsigned gpr) {
+template <bool ADJ>
+__global__ void __launch_bounds__(kSmallThreads) k_small_f32k(const SweepArgs A, unsigned gblocks, unsigned gpr,
+                                                              float* acc_a, float* acc_b) {
     pdl_trigger();
     if (blockIdx.x < gblocks) {
         pdl_wait();
@@ -61,13 +66,26 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_f32k(const SweepArgs A,
     const float hl = H[-1], hr = H[4];
     const lo_t cl = C[-1], cr = C[4];
     const float4 d = *reinterpret_cast<const float4*>((const float*)A.dlt + q);
-    const float4 r = *reinterpret_cast<const float4*>((const float*)A.rho + q);
-    group_update_store(L, A.B, A.nu2f, i0, j, k, q, hc, lo_decode4(hc, cc), hl, lo_decode(hl, cl), hr, lo_decode(hr, cr),
+    const float4 lc = lo_decode4(hc, cc);
+    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ADJ) {
+        float4 a = *reinterpret_cast<const float4*>(acc_a + q), b = *reinterpret_cast<const float4*>(acc_b + q);
+        accumulate_f32k(a.x, b.x, hc.x, lc.x);
+        accumulate_f32k(a.y, b.y, hc.y, lc.y);
+        accumulate_f32k(a.z, b.z, hc.z, lc.z);
+        accumulate_f32k(a.w, b.w, hc.w, lc.w);
+        *reinterpret_cast<float4*>(acc_a + q) = a;  // beyond nx: the row's padding, as the loads
+        *reinterpret_cast<float4*>(acc_b + q) = b;
+    } else {
+        r = *reinterpret_cast<const float4*>((const float*)A.rho + q);
+    }
+    group_update_store(L, A.B, A.nu2f, i0, j, k, q, hc, lc, hl, lo_decode(hl, cl), hr, lo_decode(hr, cr),
                        hs, hn, lo_decode4(hs, cs), lo_decode4(hn, cn), hm, hp, lo_decode4(hm, cm), lo_decode4(hp, cp), d,
                        r, (float*)A.hi_n, (lo_t*)A.lo_n, (float*)A.dlt);
 }
 
-__global__ void __launch_bounds__(kSmallThreads) k_small_f64(const SweepArgs A, unsigned gblocks, unsigned gpr) {
+template <bool ADJ>
+__global__ void __launch_bounds__(kSmallThreads) k_small_f64(const SweepArgs A, unsigned gblocks, unsigned gpr, double* acc) {
     pdl_trigger();
     if (blockIdx.x < gblocks) {
         pdl_wait();
@@ -82,8 +100,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_f64(const SweepArgs A, 
     const long long q = L.at(i, j, k);
     const double* p = (const double*)A.hi_c + q;
     double* o = (double*)A.hi_n;
-    const double v = f64_update<false>(p[-1], p[1], p[-L.pitch], p[L.pitch], p[-L.plane], p[L.plane], p[0], o[q],
-                                       ((const double*)A.rho)[q], A.nu2);
+    const double c = p[0];
+    const double v = f64_update<false>(p[-1], p[1], p[-L.pitch], p[L.pitch], p[-L.plane], p[L.plane], c, o[q],
+                                       ADJ ? 0.0 : ((const double*)A.rho)[q], A.nu2);
+    if (ADJ) acc[q] = __dadd_rn(acc[q], c);
     if (!idx_ok(q, 1, L.elems, A.B.err)) return;
     o[q] = v;
     if (A.B.periodic) {
@@ -97,20 +117,23 @@ __global__ void __launch_bounds__(kSmallThreads) k_small_f64(const SweepArgs A, 
 
 }  // namespace
 
-// one sub-step cur -> 1 - cur of a small grid, all face ghosts included
-int launch_step_small(hg_grid* g) {
+// One sub-step cur -> 1 - cur of a small grid, all face ghosts included.  With acc_a the grid is an adjoint's shadow state
+// (its source is zero and is not read) and level n is added to the running sum (acc_a, acc_b) on the way.
+int launch_step_small(hg_grid* g, void* acc_a, void* acc_b) {
     const SweepArgs A = sweep_args(g, g->zb);
     const int width = g->prec == HG_PREC_F32K ? 4 : 1;
     const unsigned gpr = (unsigned)((g->nx + width - 1) / width);
     const unsigned groups = gpr * (unsigned)g->ny * (unsigned)g->nz;
     const unsigned gblocks = A.B.faces ? (unsigned)((A.B.off[6] + kSmallThreads - 1) / kSmallThreads) : 0u;
-    const unsigned blocks = gblocks + (groups + kSmallThreads - 1) / kSmallThreads;
+    const dim3 blocks(gblocks + (groups + kSmallThreads - 1) / kSmallThreads), threads(kSmallThreads);
     int rc = prof_begin(g);
     if (rc) return rc;
     if (width == 4)
-        rc = launch_pdl(k_small_f32k, dim3(blocks), dim3(kSmallThreads), 0, g->stream, A, gblocks, gpr);
+        rc = launch_pdl(acc_a ? k_small_f32k<true> : k_small_f32k<false>, blocks, threads, 0, g->stream, A, gblocks, gpr,
+                        (float*)acc_a, (float*)acc_b);
     else
-        rc = launch_pdl(k_small_f64, dim3(blocks), dim3(kSmallThreads), 0, g->stream, A, gblocks, gpr);
+        rc = launch_pdl(acc_a ? k_small_f64<true> : k_small_f64<false>, blocks, threads, 0, g->stream, A, gblocks, gpr,
+                        (double*)acc_a);
     if (rc) return rc;
     HG_LAUNCHED("small-grid sub-step kernel");
     return prof_end(g);

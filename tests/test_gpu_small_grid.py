@@ -54,3 +54,23 @@ def test_small_slab_leaves_its_interface_ghosts_alone(prec):
         out.append(g.phi_ghosted())
         g.free()
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1), (5, 7, 3), (130, 9, 6)])
+@pytest.mark.parametrize("bc", ["dirichlet", "robin", "periodic"])
+@pytest.mark.parametrize("prec", ["f32k", "f64"])
+def test_small_adjoint_sum_is_linear_and_exact_for_one_step(prec, bc, shape):
+    """The reverse sub-step adds level m to the running sum on the way.  One reverse step sums the injection alone:
+    dL/drho = -(c dt)^2 4 pi G (lambda - mean if periodic); doubling the injection doubles a longer run's gradient
+    exactly (a power of two commutes with every rounding)."""
+    nx, ny, nz = shape
+    h = 1.0 / 64
+    dt = (robin_cfl(nx, ny, nz, h) if bc == "robin" else 0.5) * h / np.sqrt(3.0)
+    g = hg.Grid(nx, ny, nz, h, (-0.5 * nx * h, -0.5 * ny * h, -0.5 * nz * h), 1.0, 1.0, dt, prec, bc)
+    lam = I.noise(shape[::-1], 321, -1.0, 1.0).astype(np.float32).astype(np.float64)
+    one = g.adjoint(torch.from_numpy(lam).cuda(), 1).cpu().numpy()
+    want = -(dt * dt) * 4 * np.pi * (lam - (lam.mean() if bc == "periodic" else 0.0))
+    assert np.abs(one - want).max() <= 4e-16 * dt * dt * 4 * np.pi
+    a, b = (g.adjoint(torch.from_numpy(f * lam).cuda(), 7).cpu().numpy() for f in (1.0, 2.0))
+    assert np.array_equal(2.0 * a, b)
+    g.free()
