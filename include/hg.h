@@ -132,9 +132,9 @@ int hg_step(hg_grid* g, int n_substeps);
 int hg_set_temporal_depth(hg_grid* g, int k);
 int hg_set_temporal_exact(hg_grid* g, int exact);
 
-/* z planes per thread block of the single-sweep kernel (a tuning knob: more blocks and more z warm-up below, fewer
- * and longer blocks above); 0 restores the built-in rule (under which a small grid's sub-step runs without z-marching
- * blocks).  Results do not depend on it. */
+/* z planes per thread block of the compensated-float single sweep's z-marching kernel (a tuning knob: more blocks and
+ * more z warm-up below, fewer and longer blocks above); 0 restores the built-in rule, under which small grids do not march
+ * at all.  FP64 sub-steps never march.  Results do not depend on it. */
 int hg_set_block_depth(hg_grid* g, int planes);
 
 /*
@@ -260,25 +260,25 @@ void hg_free(hg_grid* g);
 
 /*
  * Batches: many independent grids (any sizes, both precisions, any boundary conditions) advanced together.  Every
- * sub-step of all grids is one batched kernel launch (plus one batched ghost-copy launch if some grid is periodic);
+ * sub-step of all grids is one batched kernel launch (two if some are large float grids, or in split mode);
  * hg_batch_step records its n sub-steps once as a CUDA graph and replays it with one graph launch, on a stream of
  * the batch that is ordered after, and before, the grids' own stream.  Results are bit-identical to hg_step on each
- * grid (single sweeps: the grids' temporal depth is not used here).  The first hg_batch_step autotunes the z extent
- * of a block by timing its first sub-steps (all candidates compute the same result) and caches the choice per
+ * grid (single sweeps: the grids' temporal depth is not used here).  The first hg_batch_step autotunes the
+ * launch by timing its first sub-steps (all candidates compute the same result) and caches the choice per
  * device and set of grid shapes for the process.  All grids must live on one device and share one stream; a grid
  * may belong to several batches and may also be stepped on its own between batch steps.
  */
 typedef struct hg_batch hg_batch;
 int hg_batch_create(hg_grid* const* grids, int n, hg_batch** b);
 int hg_batch_step(hg_batch* b, int n_substeps);
-/* autotuned FP64 z planes per block (0 before the first hg_batch_step) and blocks per batched sub-step launch */
+/* z planes per FP64 block (0 before the first hg_batch_step, then 1: its blocks do not march) and blocks per batched
+ * sub-step */
 int hg_batch_info(const hg_batch* b, int* z_planes_per_block, long long* blocks_per_substep);
-/* the whole autotuned launch: out[0] = FP64 z planes per block, out[1] = FP64 tile rows (0: per grid, 128- or
- * 32-cell rows, whichever leaves fewer lanes idle; 4: 128-cell rows for every grid), out[2] = compensated-float
- * (TMA-staged) z planes per block, out[3] = 1 when the two precisions run as separate launches per sub-step (two
- * independent chains on two streams; 0: one launch holds both).  The choice is timed on the first sub-steps of the
- * first hg_batch_step and cached per device and set of grids for the life of the process (an autotuner of this
- * library; the paper has no counterpart). */
+/* the whole autotuned launch: out[0] = z planes per FP64 block, out[1] = 0 (no FP64 tile rows: cells are numbered flat),
+ * out[2] = z planes per block of the float grids too large for that (TMA-staged), out[3] = 1 when the two precisions
+ * run as separate launches per sub-step (two independent chains on two streams; 0: one launch holds both).  The choice
+ * is timed on the first sub-steps of the first hg_batch_step and cached per device and set of grids for the life of
+ * the process (an autotuner of this library; the paper has no counterpart). */
 int hg_batch_tuning(const hg_batch* b, int out[4]);
 /* Pin the launch mode instead of letting the autotuner choose it: mode 1 = split (one launch per precision class per
  * sub-step, two streams), 0 = one launch for both, -1 = autotuned (the default).  The other knobs are still tuned, on

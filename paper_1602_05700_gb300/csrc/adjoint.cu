@@ -58,31 +58,22 @@ __global__ void __launch_bounds__(kThreads) k_inject(const T* __restrict__ v, vo
     });
 }
 
-// acc += lambda^m on the interior, for grids whose sub-step does not do it on the way (stencil_small.cu).  All three
-// arrays are padded, so groups of 4 (rows have room for the last one) whatever nx is.
-template <bool F64>
-__global__ void __launch_bounds__(kThreads) k_accumulate(const void* hi, const void* lo, void* acc_a, void* acc_b, Layout L,
+// acc += lambda^m on the interior, for the float grids whose sub-step does not do it on the way (flat_sweep, stencil.cu).
+// All arrays are padded, so groups of 4 (rows have room for the last one) whatever nx is.
+__global__ void __launch_bounds__(kThreads) k_accumulate(const float* __restrict__ hi, const lo_code* __restrict__ lo,
+                                                         float* __restrict__ acc_a, float* __restrict__ acc_b, Layout L,
                                                          unsigned gpr) {
     for (long long t = blockIdx.x * (long long)kThreads + threadIdx.x; t < (long long)gpr * L.ny * L.nz;
          t += (long long)gridDim.x * kThreads) {
         const long long row = t / gpr;
         const long long q = L.at((int)(t - row * gpr) * 4, (int)(row % L.ny), (int)(row / L.ny));
-        if constexpr (F64) {
-            Vec<double, 4> a = ldv<double, 4>((double*)acc_a + q);
-            const Vec<double, 4> x = ldv<double, 4>((const double*)hi + q);
+        Vec<float, 4> a = ldv<float, 4>(acc_a + q), b = ldv<float, 4>(acc_b + q);
+        const Vec<float, 4> h = ldv<float, 4>(hi + q);
+        const Vec<lo_code, 4> c = ldv<lo_code, 4>(lo + q);
 #pragma unroll
-            for (int e = 0; e < 4; ++e) a.v[e] += x.v[e];
-            stv<double, 4>((double*)acc_a + q, a);
-        } else {
-            Vec<float, 4> a = ldv<float, 4>((float*)acc_a + q), b = ldv<float, 4>((float*)acc_b + q);
-            const Vec<float, 4> h = ldv<float, 4>((const float*)hi + q);
-            const Vec<lo_code, 4> c = ldv<lo_code, 4>((const lo_code*)lo + q);
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                accumulate_f32k(a.v[e], b.v[e], h.v[e], lo_decode(h.v[e], __ushort_as_half(c.v[e])));
-            stv<float, 4>((float*)acc_a + q, a);
-            stv<float, 4>((float*)acc_b + q, b);
-        }
+        for (int e = 0; e < 4; ++e) accumulate_f32k(a.v[e], b.v[e], h.v[e], lo_decode(h.v[e], __ushort_as_half(c.v[e])));
+        stv<float, 4>(acc_a + q, a);
+        stv<float, 4>(acc_b + q, b);
     }
 }
 
@@ -151,10 +142,8 @@ int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b) {
     const unsigned gpr = (unsigned)((a->nx + 3) / 4);
     const long long n = ((long long)gpr * a->ny * a->nz + kThreads - 1) / kThreads;
     const unsigned blocks = (unsigned)(n < (1LL << 22) ? n : 1LL << 22);
-    if (a->prec == HG_PREC_F64)
-        k_accumulate<true><<<blocks, kThreads, 0, a->stream>>>(a->phi[a->cur], nullptr, acc_a, acc_b, a->L, gpr);
-    else
-        k_accumulate<false><<<blocks, kThreads, 0, a->stream>>>(a->phi[a->cur], a->lo[a->cur], acc_a, acc_b, a->L, gpr);
+    k_accumulate<<<blocks, kThreads, 0, a->stream>>>((const float*)a->phi[a->cur], (const lo_code*)a->lo[a->cur],
+                                                     (float*)acc_a, (float*)acc_b, a->L, gpr);
     HG_LAUNCHED("adjoint accumulation kernel");
     return HG_OK;
 }

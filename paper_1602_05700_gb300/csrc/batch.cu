@@ -1,26 +1,23 @@
 // Many independent grids advanced together (the batching workload: uneven sizes, mixed precisions).
 //
-// One sub-step of every grid is one batched kernel launch (stencil.cu, k_step_batch: block -> grid by a prefix
-// table; compensated-float grids run the TMA-staged sweep with their tensor maps in the table, FP64 grids the
-// register-staged FP64 sweep, in the same launch, so HBM-bound and FP64-bound blocks share the SMs; boundary ghosts
-// are written inside the launch).  hg_batch_step(b, n) records the n sub-steps once as a CUDA graph on the batch's
-// own stream and replays it with a single graph launch; the kernels read the per-grid arguments from two device
-// tables (for the two time-level parities), refreshed from the grids before every replay, so the graph stays valid
-// while the grids' states move on.  Results are identical to stepping each grid on its own: the per-cell arithmetic
-// is the same code.
+// One sub-step of every grid is one batched launch of the flat sweep (stencil.cu, k_batch_flat: block -> grid by a prefix
+// table; FP64 and float blocks alternate, so that FP64- and integer-bound and HBM-bound ones share the SMs; boundary ghosts
+// are written inside the launch); float grids large enough for the TMA-staged sweep are a second launch beside it.
+// hg_batch_step(b, n) records the n sub-steps once as a CUDA graph on the batch's own stream and replays it with a
+// single graph launch; the kernels read the per-grid arguments from two device tables (for the two time-level
+// parities), refreshed from the grids before every replay, so the graph stays valid while the grids' states move on.
+// Results are identical to stepping each grid on its own: the per-cell arithmetic is the same code.
 //
-// Autotuning: three knobs of the launch are chosen by timing the first sub-steps of the first hg_batch_step with
-// CUDA events -- every candidate computes the same result, so the timing runs are real sub-steps -- and cached per
+// 48 grids of 64^3 to 192^3, alternating precisions, per sub-step: 2.18 ms with marching FP64 blocks and TMA-staged float
+// blocks in one launch (the FP64 half latency-bound at 16 warps per SM, 60% of a 96-cell row's tile in use), see
+// sweep_flat.cuh for what the flat sweep changes.
+//
+// Autotuning: two knobs of the launch are chosen by timing the first sub-steps of the first hg_batch_step with CUDA
+// events -- every candidate computes the same result, so the timing runs are real sub-steps -- and cached per
 // (device, set of grid shapes/precisions/boundaries) for the process:
-//   * the tile shape of an FP64 block: rows of 128 cells (4 per lane) for every grid, or per grid whichever of
-//     128- and 32-cell rows (1 per lane) leaves fewer lanes idle (a 96-cell row fills 75% of a 128-cell tile; the
-//     FP64 pipe pays for idle lanes, since its rate is per warp instruction);
-//   * the z extent of an FP64 block (8 .. 64 planes: the number of blocks against the share of the z warm-up);
-//   * the z extent of a TMA-staged compensated-float block (8 or 16 planes);
-//   * one launch per sub-step for both precisions, or two (split mode: an FP64-only launch and a float-only launch
-//     per sub-step, each with its own sweep's registers and block shape, as two independent chains on two streams).
-// All FP64 candidates are timed first (eight), then the split mode with the best FP64 setting, then the float
-// extent of 16 planes with the better of the two.
+//   * one flat launch per sub-step for both precisions, or two (split mode: an FP64 launch and a float launch per
+//     sub-step, as two independent chains on two streams);
+//   * the z extent of a TMA-staged block of the large float grids (8 or 16 planes).
 #include <stdio.h>
 #include <string.h>
 
@@ -40,21 +37,16 @@ struct hg_batch {
     int device;
     cudaStream_t stream;  // own non-blocking stream (graphs cannot be captured on the legacy default stream)
     cudaEvent_t ev_in, ev_out;
-    TmaEntry* d_tab[2];   // per-grid entries, per parity
-    unsigned* d_first;
-    unsigned total_blocks;
-    std::vector<unsigned> first;
-    int zb;    // FP64 planes per block, 0 until tuned
-    int cpl;   // FP64 cells per lane: 0 = per grid, whichever tile row fits better; 4 = 128-cell rows everywhere
-    int zb32;  // compensated-float (TMA-staged) planes per block
-    int split; // 1: FP64 and compensated-float entries as two launches per sub-step, on two streams
+    BatchEntry* d_tab[2];  // per-grid entries, per parity: FP64 grids, then float ones, then large float ones
+    unsigned* d_first;     // the three classes' prefix tables of block numbers, each with one entry more than grids
+    int n64, n32, nbig;
+    unsigned blocks64, blocks32, blocksbig;
+    int zb;    // 0 until tuned, then 1: planes of a flat block
+    int zb32;  // z planes per block of the large float grids (TMA-staged)
+    int split; // 1: FP64 and float entries as two launches per sub-step, on two streams
     int force_split;  // -1: the autotuner chooses split; 0 or 1: pinned by hg_batch_set_split
-    // split mode: the two classes' own prefix tables (FP64 entries first in the table, then the float ones)
     cudaStream_t stream2;
     cudaEvent_t ev_fork, ev_join;
-    unsigned* d_first2;  // FP64 prefix (n64 + 1 entries), then float prefix (n32 + 1 entries)
-    int n64, n32;
-    unsigned blocks64, blocks32;
     // graph of `graph_steps` sub-steps
     cudaGraph_t graph;
     cudaGraphExec_t exec;
@@ -65,7 +57,7 @@ namespace {
 
 std::mutex g_tune_mu;
 struct Tuning {
-    int zb, cpl, zb32, split;
+    int zb32, split;
 };
 std::map<std::string, Tuning> g_tuned;  // autotuner cache: key -> the chosen launch
 
@@ -85,35 +77,34 @@ std::string tune_key(const hg_batch* b) {
     return k;
 }
 
-// device tables for the sub-step that starts from parity p (0: every grid's current level, 1: the next one)
-// The table lists the FP64 grids first, largest first, then the compensated-float grids: the block scheduler hands
-// out blocks in index order, so the long FP64-bound blocks start first and the short HBM-bound ones fill in around
-// them and make up the tail of each launch.
+// FP64 grids, float grids of the flat sweep, large float grids; largest first within a class
+int class_of(const hg_grid* g) { return g->prec == HG_PREC_F64 ? 0 : flat_sized(g) ? 1 : 2; }
 std::vector<hg_grid*> launch_order(const hg_batch* b) {
     std::vector<hg_grid*> o(b->grids);
     auto cells = [](const hg_grid* g) { return (long long)g->nx * g->ny * g->nz; };
     std::stable_sort(o.begin(), o.end(), [&](const hg_grid* a, const hg_grid* c) {
-        const bool a64 = a->prec == HG_PREC_F64, c64 = c->prec == HG_PREC_F64;
-        if (a64 != c64) return a64;
+        if (class_of(a) != class_of(c)) return class_of(a) < class_of(c);
         return cells(a) > cells(c);
     });
     return o;
 }
 
+// device tables for the sub-steps that start from parity p (0: every grid's current level, 1: the next one)
 int upload_tables(hg_batch* b) {
-    std::vector<TmaEntry> tab[2];
+    std::vector<BatchEntry> tab[2];
     const std::vector<hg_grid*> order = launch_order(b);
     for (int p = 0; p < 2; ++p) {
         for (hg_grid* g : order) {
             const int cur = g->cur;
             g->cur = cur ^ p;
-            TmaEntry e;
+            BatchEntry e;
             memset(&e, 0, sizeof e);
             int rc = HG_OK;
-            if (g->prec == HG_PREC_F32K) {
+            if (class_of(g) == 2) {
                 rc = tma_entry(g, &e, b->zb32);
             } else {
-                e.A = sweep_args(g, b->zb, b->cpl);
+                e.A = sweep_args(g, 0);
+                e.G = flat_grid(g, kBatchThreads);
                 e.err = g->derr;
             }
             g->cur = cur;
@@ -121,50 +112,49 @@ int upload_tables(hg_batch* b) {
             tab[p].push_back(e);
         }
     }
-    b->first.assign(1, 0);
-    for (const TmaEntry& e : tab[0]) b->first.push_back(b->first.back() + sweep_blocks(e.A));
-    b->total_blocks = b->first.back();
-    // the classes' own prefixes: FP64 entries are [0, n64), float entries [n64, n)
-    b->n64 = 0;
-    for (hg_grid* g : order) b->n64 += g->prec == HG_PREC_F64 ? 1 : 0;
-    b->n32 = b->n - b->n64;
-    std::vector<unsigned> first2;
-    first2.push_back(0);
-    for (int i = 0; i < b->n64; ++i) first2.push_back(first2.back() + sweep_blocks(tab[0][i].A));
-    b->blocks64 = first2.back();
-    first2.push_back(0);
-    for (int i = b->n64; i < b->n; ++i) first2.push_back(first2.back() + sweep_blocks(tab[0][i].A));
-    b->blocks32 = first2.back();
-    HG_CUDA(cudaMemcpyAsync(b->d_first2, first2.data(), first2.size() * sizeof(unsigned), cudaMemcpyHostToDevice,
-                            b->stream));
+    int n[3] = {0, 0, 0};
+    unsigned blocks[3];
+    std::vector<unsigned> first;
+    for (hg_grid* g : order) ++n[class_of(g)];
+    for (int c = 0, i = 0; c < 3; ++c) {
+        first.push_back(0);
+        for (int e = 0; e < n[c]; ++e, ++i)
+            first.push_back(first.back() + (c == 2 ? sweep_blocks(tab[0][i].A)
+                                                   : (tab[0][i].G.tiles + kBatchTiles - 1) / kBatchTiles));
+        blocks[c] = first.back();
+    }
+    b->n64 = n[0], b->n32 = n[1], b->nbig = n[2];
+    b->blocks64 = blocks[0], b->blocks32 = blocks[1], b->blocksbig = blocks[2];
     for (int p = 0; p < 2; ++p)
-        HG_CUDA(cudaMemcpyAsync(b->d_tab[p], tab[p].data(), tab[p].size() * sizeof(TmaEntry), cudaMemcpyHostToDevice,
+        HG_CUDA(cudaMemcpyAsync(b->d_tab[p], tab[p].data(), tab[p].size() * sizeof(BatchEntry), cudaMemcpyHostToDevice,
                                 b->stream));
-    HG_CUDA(cudaMemcpyAsync(b->d_first, b->first.data(), b->first.size() * sizeof(unsigned), cudaMemcpyHostToDevice,
-                            b->stream));
+    HG_CUDA(cudaMemcpyAsync(b->d_first, first.data(), first.size() * sizeof(unsigned), cudaMemcpyHostToDevice, b->stream));
     HG_CUDA(cudaStreamSynchronize(b->stream));  // the host vectors go out of scope
     return HG_OK;
 }
 
-// the launches of `count` sub-steps, the first of parity p0.  Split mode: the FP64 chain on the batch stream and
-// the float chain on the second stream, forked from and joined back into the batch stream (the chains touch
-// different grids, so they need no ordering between them).
+// The launches of `count` sub-steps, the first of parity p0.  The second stream, forked from and joined back into the
+// batch stream, carries the large float grids and in split mode every float grid (the chains touch different grids, so
+// they need no ordering between them).
 int enqueue_substeps(hg_batch* b, int p0, int count) {
     int rc = HG_OK;
-    if (!b->split) {
-        for (int s = 0; s < count && rc == HG_OK; ++s)
-            rc = launch_step_batch(b->stream, b->d_tab[(p0 + s) & 1], b->d_first, b->n, b->total_blocks);
-        return rc;
+    const bool second = b->nbig > 0 || (b->split && b->n32 > 0);
+    if (second) {
+        HG_CUDA(cudaEventRecord(b->ev_fork, b->stream));
+        HG_CUDA(cudaStreamWaitEvent(b->stream2, b->ev_fork, 0));
     }
-    HG_CUDA(cudaEventRecord(b->ev_fork, b->stream));
-    HG_CUDA(cudaStreamWaitEvent(b->stream2, b->ev_fork, 0));
+    const unsigned *f64 = b->d_first, *f32 = f64 + b->n64 + 1, *fbig = f32 + b->n32 + 1;
     for (int s = 0; s < count && rc == HG_OK; ++s) {
-        const int p = (p0 + s) & 1;
-        rc = launch_batch_class(b->stream, true, b->d_tab[p], b->d_first2, b->n64, b->blocks64);
-        if (rc == HG_OK)
-            rc = launch_batch_class(b->stream2, false, b->d_tab[p] + b->n64, b->d_first2 + b->n64 + 1, b->n32,
-                                    b->blocks32);
+        const BatchEntry *t64 = b->d_tab[(p0 + s) & 1], *t32 = t64 + b->n64, *tbig = t32 + b->n32;
+        if (b->split) {
+            rc = launch_batch_flat(b->stream, t64, f64, b->n64, b->blocks64, t32, f32, 0, 0u);
+            if (rc == HG_OK) rc = launch_batch_flat(b->stream2, t64, f64, 0, 0u, t32, f32, b->n32, b->blocks32);
+        } else {
+            rc = launch_batch_flat(b->stream, t64, f64, b->n64, b->blocks64, t32, f32, b->n32, b->blocks32);
+        }
+        if (rc == HG_OK) rc = launch_batch_tma(b->stream2, tbig, fbig, b->nbig, b->blocksbig);
     }
+    if (!second) return rc;
     // join even after an error, so that a capture in progress ends with both streams in it
     cudaError_t e1 = cudaEventRecord(b->ev_join, b->stream2);
     cudaError_t e2 = cudaStreamWaitEvent(b->stream, b->ev_join, 0);
@@ -190,25 +180,21 @@ int autotune(hg_batch* b, int budget, int* taken) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tuned.find(key);
         if (it != g_tuned.end()) {
-            b->zb = it->second.zb;
-            b->cpl = it->second.cpl;
+            b->zb = 1;
             b->zb32 = it->second.zb32;
             b->split = it->second.split;
             return upload_tables(b);
         }
     }
-    bool any64 = false, any32 = false;
+    bool any64 = false, any32 = false, anybig = false;
     for (hg_grid* g : b->grids) {
-        any64 = any64 || g->prec == HG_PREC_F64;
-        any32 = any32 || g->prec == HG_PREC_F32K;
+        any64 = any64 || class_of(g) == 0;
+        any32 = any32 || class_of(g) == 1;
+        anybig = anybig || class_of(g) == 2;
     }
     std::vector<Tuning> cand;
-    const int split0 = b->force_split > 0 ? 1 : 0;
-    if (any64)
-        for (int cpl : {0, 4})
-            for (int zb : {8, 16, 32, 64}) cand.push_back({zb, cpl, 8, split0});
-    else
-        cand.push_back({8, 0, 8, split0});
+    cand.push_back({8, b->force_split > 0 ? 1 : 0});
+    if (b->force_split < 0 && any64 && any32) cand.push_back({8, 1});
     Tuning best = cand[0];
     float best_ms = -1.f;
     cudaEvent_t e0, e1;
@@ -221,8 +207,6 @@ int autotune(hg_batch* b, int budget, int* taken) {
             complete = false;
             return false;
         }
-        b->zb = t.zb;
-        b->cpl = t.cpl;
         b->zb32 = t.zb32;
         b->split = t.split;
         if ((rc = upload_tables(b))) return false;
@@ -246,12 +230,7 @@ int autotune(hg_batch* b, int budget, int* taken) {
     };
     for (const Tuning& t : cand)
         if (!time_one(t)) break;
-    if (rc == HG_OK && complete && best_ms >= 0.f && b->force_split < 0) {  // each class as a launch of its own
-        Tuning t = best;
-        t.split = 1;
-        time_one(t);
-    }
-    if (rc == HG_OK && complete && any32 && best_ms >= 0.f) {
+    if (rc == HG_OK && complete && anybig && best_ms >= 0.f) {
         Tuning t = best;
         t.zb32 = 16;
         time_one(t);
@@ -259,16 +238,8 @@ int autotune(hg_batch* b, int budget, int* taken) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
-    if (best_ms < 0.f) {  // no budget to tune: the default launch this time
-        b->zb = 8;
-        b->cpl = 0;
-        b->zb32 = 8;
-        b->split = split0;
-        return upload_tables(b);
-    }
-    b->zb = best.zb;
-    b->cpl = best.cpl;
-    b->zb32 = best.zb32;
+    b->zb = 1;
+    b->zb32 = best.zb32;  // without the budget to time anything, the first candidate
     b->split = best.split;
     if (complete) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -287,7 +258,7 @@ void destroy_graph(hg_batch* b) {
 
 void release(hg_batch* b) {
     destroy_graph(b);
-    void* ptrs[] = {b->d_tab[0], b->d_tab[1], b->d_first, b->d_first2};
+    void* ptrs[] = {b->d_tab[0], b->d_tab[1], b->d_first};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     cudaEvent_t evs[] = {b->ev_in, b->ev_out, b->ev_fork, b->ev_join};
@@ -329,9 +300,8 @@ int hg_batch_create(hg_grid* const* grids, int n, hg_batch** out) {
     ck(cudaStreamCreateWithFlags(&b->stream2, cudaStreamNonBlocking), "cudaStreamCreate");
     for (cudaEvent_t* ev : {&b->ev_in, &b->ev_out, &b->ev_fork, &b->ev_join})
         ck(cudaEventCreateWithFlags(ev, cudaEventDisableTiming), "cudaEventCreate");
-    for (int p = 0; p < 2 && rc == HG_OK; ++p) ck(cudaMalloc(&b->d_tab[p], n * sizeof(TmaEntry)), "cudaMalloc(table)");
-    ck(cudaMalloc(&b->d_first, (n + 1) * sizeof(unsigned)), "cudaMalloc(table)");
-    ck(cudaMalloc(&b->d_first2, (n + 2) * sizeof(unsigned)), "cudaMalloc(table)");
+    for (int p = 0; p < 2 && rc == HG_OK; ++p) ck(cudaMalloc(&b->d_tab[p], n * sizeof(BatchEntry)), "cudaMalloc(table)");
+    ck(cudaMalloc(&b->d_first, (n + 3) * sizeof(unsigned)), "cudaMalloc(table)");
     if (rc == HG_OK) rc = upload_tables(b);
     if (rc != HG_OK) {
         release(b);
@@ -401,7 +371,7 @@ int hg_batch_info(const hg_batch* b, int* z_planes_per_block, long long* blocks_
     HG_RANGE("hg_batch_info");
     if (!b) return fail(HG_ERR_ARG, "null batch");
     if (z_planes_per_block) *z_planes_per_block = b->zb;
-    if (blocks_per_substep) *blocks_per_substep = b->total_blocks;
+    if (blocks_per_substep) *blocks_per_substep = (long long)b->blocks64 + b->blocks32 + b->blocksbig;
     return HG_OK;
 }
 
@@ -409,7 +379,7 @@ int hg_batch_tuning(const hg_batch* b, int out[4]) {
     HG_RANGE("hg_batch_tuning");
     if (!b || !out) return fail(HG_ERR_ARG, "null argument");
     out[0] = b->zb;
-    out[1] = b->cpl;
+    out[1] = 0;
     out[2] = b->zb32;
     out[3] = b->split;
     return HG_OK;

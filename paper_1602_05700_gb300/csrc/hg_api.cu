@@ -773,8 +773,8 @@ int hg_adjoint_step(hg_grid* g, int n_substeps) {
     if (n_substeps < 0) return fail(HG_ERR_ARG, "n_substeps must be >= 0");
     hg_grid* a = g->adj;
     for (int s = 0; s < n_substeps; ++s) {
-        if (small_grid(a)) {  // the sum rides in the sub-step
-            if ((rc = launch_step_small(a, g->acc[0], g->acc[1]))) return rc;
+        if (flat_sweep(a)) {  // the sum rides in the sub-step
+            if ((rc = launch_step_flat(a, g->acc[0], g->acc[1]))) return rc;
         } else {
             if ((rc = adjoint_accumulate(a, g->acc[0], g->acc[1]))) return rc;
             if ((rc = launch_step_single(a))) return rc;

@@ -246,8 +246,11 @@ int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cud
 
 // kernels' host launchers (each returns HG_OK or an error code)
 int launch_step_single(hg_grid* g);                  // one sub-step: cur -> 1-cur, all ghosts (stencil.cu)
-bool small_grid(const hg_grid* g);                   // whether launch_step_small serves this grid (stencil.cu)
-int launch_step_small(hg_grid* g, void* acc_a = nullptr, void* acc_b = nullptr);  // a small grid's (stencil_small.cu)
+bool flat_sized(const hg_grid* g);                   // whether the flat sweep is the faster one for this grid (stencil.cu)
+bool flat_sweep(const hg_grid* g);                   // whether launch_step_flat serves its single sub-steps
+// one sub-step by the flat sweep; with acc_a, g is an adjoint's shadow state (zero source) and its level n is added to the
+// running sum (acc_a, acc_b) on the way (stencil_flat.cu)
+int launch_step_flat(hg_grid* g, void* acc_a = nullptr, void* acc_b = nullptr);
 int adjoint_inject(hg_grid* a, const void* v, int vdt);
 int adjoint_accumulate(hg_grid* a, void* acc_a, void* acc_b);
 int adjoint_gradient(hg_grid* a, const void* acc_a, const void* acc_b, void* out, int odt, double* scratch);
@@ -282,7 +285,7 @@ int prof_fold(hg_grid* g);   // synchronise and add the recorded pairs to prof_m
 
 // ---- sweep arguments (stencil.cu) ----
 struct Bnd {
-    int faces;              // 1: Robin ghosts to update (block epilogue)
+    int faces;              // 1: Robin ghosts to update
     int periodic;           // 1: the sweep stores the new boundary cells into the opposite ghosts too
     int zskip;              // bit 0 / bit 1: the -z / +z face is an interface to a neighbouring slab (its ghost
                             // plane is supplied by the caller before each sub-step and never written by a sweep)
@@ -291,6 +294,18 @@ struct Bnd {
     long long off[7];       // face offsets in the ghost enumeration (hg::Faces)
     int* err;               // the grid's device error word (debug index checks)
 };
+
+// n / d for n < 2^31 by one multiplication: with l = ceil(log2 d) and mul = ceil(2^(31+l) / d) < 2^32 the error n (mul d -
+// 2^(31+l)) stays below 2^(31+l), so (n mul) >> (31 + l) is the quotient
+struct FastDiv {
+    unsigned d, mul, shr;
+    __device__ __forceinline__ unsigned div(unsigned n) const { return __umulhi(n + n, mul) >> shr; }
+};
+inline FastDiv fast_div(unsigned d) {
+    unsigned l = 0;
+    while ((1ull << l) < d) ++l;
+    return {d, (unsigned)(((1ull << (31 + l)) + d - 1) / d), l};
+}
 
 // Everything one sweep of one grid needs (a launch of one grid, or one entry of a batched launch).
 struct SweepArgs {
@@ -306,29 +321,40 @@ struct SweepArgs {
     int zb;            // z planes per block
     int prec;
     int exact;         // fused sub-steps: inner levels round their compensation as a store and a load would
-    int cpl;           // FP64 sweep: x cells per lane (4: 128-cell tile rows; 1: 32-cell rows, for nx that 128 fits badly)
     unsigned gx, gy;   // blocks in x and y of this grid's sweep
     Bnd B;
 };
 
-SweepArgs sweep_args(const hg_grid* g, int zb, int cpl = 0);  // sub-step cur -> 1 - cur of grid g; zb = 0: default z
-                                                              // chunk; cpl = 0: FP64 cells per lane by tile fit
-int f64_cells_per_lane(int nx);  // 4, or 1 when 32-cell tile rows waste fewer lanes than 128-cell ones
+SweepArgs sweep_args(const hg_grid* g, int zb);  // sub-step cur -> 1 - cur of grid g; zb = 0: default z chunk (TMA sweep)
+
+// The tiles of a flat sweep (sweep_flat.cuh) with a given number of threads per block
+struct FlatGrid {
+    unsigned ghost_tiles, tiles;  // Robin ghosts first, then per_plane.d tiles for each plane
+    FastDiv per_plane, gpr;       // tiles per plane, groups per row
+    int wide;                     // a plane holds 2^31 groups or more
+};
+FlatGrid flat_grid(const hg_grid* g, int threads);
+
 // a 3-D TMA map over a padded array (pitch x (ny+2) x (nz+2) elements of `bytes` each), boxes box_x x box_y x 1
 int tma_encode(CUtensorMap* m, void* base, const Layout& L, int bytes, int box_x, int box_y);
 
-// One grid of a batched launch: its sweep arguments and, for a compensated-float grid, the tensor maps of its state
-// (hi, lo codes, dlt, s of level n) and its error word.
-struct alignas(128) TmaEntry {
+// One grid of a batched launch: its sweep arguments, its tiles (flat sweep) or the tensor maps of its state (TMA sweep: hi, lo
+// codes, dlt, s of level n), and its error word.
+struct alignas(128) BatchEntry {
     CUtensorMap m[4];
     SweepArgs A;
+    FlatGrid G;
     int* err;
 };
-int tma_entry(hg_grid* g, TmaEntry* e, int zb = 0);  // compensated-float g's sub-step cur -> 1 - cur (all ghosts in the launch)
-int launch_step_batch(cudaStream_t st, const TmaEntry* tab, const unsigned* first, int n, unsigned total_blocks);
-// one precision class of a batched sub-step (FP64 entries, or compensated-float entries) as a launch of its own
-int launch_batch_class(cudaStream_t st, bool f64, const TmaEntry* tab, const unsigned* first, int n,
-                       unsigned total_blocks);
+constexpr int kBatchThreads = 128;  // threads of a flat batched block
+constexpr int kBatchTiles = 4;      // tiles it takes, one after the other
+int tma_entry(hg_grid* g, BatchEntry* e, int zb = 0);  // large float g's sub-step cur -> 1 - cur (all ghosts in the launch)
+// a batched sub-step of n64 FP64 and n32 float entries by the flat sweep in one launch (either may be 0): block ranges
+// first64 / first32 (prefix tables), blocks64 / blocks32 blocks
+int launch_batch_flat(cudaStream_t st, const BatchEntry* tab64, const unsigned* first64, int n64, unsigned blocks64,
+                      const BatchEntry* tab32, const unsigned* first32, int n32, unsigned blocks32);
+// the large float entries of a batched sub-step, by the TMA sweep
+int launch_batch_tma(cudaStream_t st, const BatchEntry* tab, const unsigned* first, int n, unsigned blocks);
 unsigned sweep_blocks(const SweepArgs& A);
 
 // ---- deterministic reductions --------------------------------------------------------------------------------

@@ -1,19 +1,21 @@
 // The FP64 Laplacian sum of the sub-step, L = (((((xl-c) + (xr-c)) + (ys-c)) + (yn-c)) + (zm-c)) + (zp-c) with
 // every difference and every partial sum rounded to double (the plain evaluation order of Eq. HNeq's discretisation,
-// Sec. 2), computed with integer instructions where no rounding of that order changes anything.
+// Sec. 2), computed with integer instructions that give the same bits.
 //
-// Why: GB300 executes FP64 arithmetic at about 2 operations per SM per clock, while its integer pipes take 64 lanes
-// per clock; the 11 FP64 operations of L are most of an FP64 sub-step's 15.  When they are all exact, their result is
-// the exact sum of the six differences, which integers give bit for bit.
+// Why: GB300 executes FP64 arithmetic at about 2 operations per SM and clock (16 cycles per warp instruction), while
+// its integer pipes take 64 lanes per clock; the 11 FP64 operations of L are most of an FP64 sub-step's 15.
 //
-// When every operation is exact: write each value as sign * M * 2^(e - 1075) (M the 53-bit significand, e the biased
-// exponent).  If c is normal with 64 <= e_c <= 2000 and each neighbour x has c's sign and an exponent within one of
-// e_c, then |x| and |c| are integers X, C in units u = 2^(e_c - 1 - 1075), and x - c = sgn(c) (X - C) u exactly.  If
-// also |X - C| < 2^50 for all six, every difference and every partial sum is an integer below 6 * 2^50 < 2^53 in
-// units of u (u >= 2^-1012, a normal number), hence representable: IEEE subtraction and addition return them
-// exactly, and L = sgn(c) S u with S the integer sum (an exact zero being +0, as x - x and a + (-a) are in
-// round-to-nearest).  A cell and six neighbours that are all +0 give L = +0 as well.  Otherwise lap6_int returns
-// false and the caller evaluates the FP64 order itself.
+// Units: let e be the smallest biased exponent of the seven values and u = 2^(e - 1075) its unit in the last place.  If all
+// seven have one sign, 64 <= e <= 1993 and no exponent exceeds e + 7, each value is an integer below 2^60 times u, so
+// every difference and every sum of differences is an exact integer below 2^63, and u >= 2^-1011 keeps every
+// rounded result normal.  An operation of the FP64 order is then the rounding of an exact integer to 53 significant
+// bits, to nearest even:
+//   * an integer of magnitude at most 2^53 is unchanged.  Where that holds for all six differences and all five partial
+//     sums (any field whose neighbours lie within a factor of about two: potentials, and the steep tails of compact
+//     sources too), L is the plain integer sum;
+//   * otherwise each operation is rounded as it is made (round53).
+// A zero result is +0, as x - x and a + (-a) are in round-to-nearest.  A cell and six neighbours that are all +0 give
+// L = +0 as well.  Other stencils (sign changes, exponents further apart, subnormals) are left to FP64.
 #pragma once
 
 #ifndef __CUDACC__
@@ -58,120 +60,124 @@ __host__ __device__ __forceinline__ int clz64(unsigned long long v) {
 #endif
 }
 
-// The steep regions (neighbours up to a factor of 2 from c, as in the tails of a compact source) fail the 2^50 bound,
-// but there each difference x - c is still exact (Sterbenz: c/2 <= x <= 2c of one sign), only the partial sums
-// round: the six differences come from integers -- the same units, the bound replaced by the Sterbenz condition
-// 2X >= C and X <= 2C -- and only the five additions remain for the FP64 unit.
-//
-// lap6_exact_sum evaluates the first condition (every operation of L exact; its S is then L in units of u) and
-// lap6_exact_diffs the second (every difference exact), each in one pass over the six neighbours.  A stencil that
-// passes the first passes the second, and a stencil of seven +0 passes both (L = +0, every difference +0).
-struct Lap6Sum {
-    long long S;  // sum of the six differences in units u = 2^(e_c - 1076), meaningful when exact
-    bool exact;
+__host__ __device__ __forceinline__ unsigned umin3(unsigned a, unsigned b, unsigned c) {
+#ifdef __CUDA_ARCH__
+    return __vimin3_u32(a, b, c);
+#else
+    const unsigned m = a < b ? a : b;
+    return m < c ? m : c;
+#endif
+}
+__host__ __device__ __forceinline__ unsigned umax3(unsigned a, unsigned b, unsigned c) {
+#ifdef __CUDA_ARCH__
+    return __vimax3_u32(a, b, c);
+#else
+    const unsigned m = a > b ? a : b;
+    return m > c ? m : c;
+#endif
+}
+
+// the significand of a double, hidden bit set, shifted left by d & 7 (on the device d is taken modulo 32 by the funnel
+// shift: only d <= 7 is used)
+__host__ __device__ __forceinline__ long long significand(unsigned long long b, unsigned d) {
+#ifdef __CUDA_ARCH__
+    const unsigned lo = (unsigned)b, hi = ((unsigned)(b >> 32) & 0xfffffu) | 0x100000u;
+    return (long long)(((unsigned long long)__funnelshift_l(lo, hi, d) << 32) | __funnelshift_l(0u, lo, d));
+#else
+    return (long long)(((b & kFrac52) | kHidden52) << (d & 7u));
+#endif
+}
+
+// the six differences in units of the stencil's smallest ulp, and which of the forms above serve it
+struct Lap6 {
+    long long D[6];
+    long long S;   // their plain sum: L in units u when `exact`
+    unsigned h;    // sign and smallest biased exponent
+    bool exact;    // no operation of the FP64 order rounds
+    bool ok;       // the integer forms hold
 };
 
-__host__ __device__ __forceinline__ long long lap_units(double x, unsigned hc, long long C, unsigned& d) {
-    const unsigned long long xb = dbits(x);
-    d = (unsigned)(xb >> 52) - hc + 1u;  // 0, 1, 2: c's sign and exponent e_c - 1 .. e_c + 1
-    return (long long)(((xb & kFrac52) | kHidden52) << (d & 3u));
+// hi word of |v|, up to one: v ^ (v >> 63), so a magnitude of at most 2^53 leaves the bits from 2^21 on clear
+__host__ __device__ __forceinline__ unsigned mag_hi(long long v) {
+    const int h = (int)(v >> 32);
+    return (unsigned)(h ^ (h >> 31));
 }
 
-// c normal in the range above, or c = +0 with six +0 neighbours (c = +0: its terms pass only for neighbours +0,
-// D = 0, or positive subnormals, D > 0, so S = 0 means every neighbour is +0 -- the quiet regions ahead of a front)
-__host__ __device__ __forceinline__ bool lap_c_ok(unsigned long long cb, long long S) {
-    const unsigned ec = (unsigned)(cb >> 52) & 0x7ffu;
-    return (ec >= 64u && ec <= 2000u) || (cb == 0ull && S == 0);
-}
-
-__host__ __device__ __forceinline__ Lap6Sum lap6_exact_sum(double c, double x0, double x1, double x2, double x3,
-                                                           double x4, double x5) {
-    const unsigned long long cb = dbits(c);
-    const unsigned hc = (unsigned)(cb >> 52);  // sign and biased exponent of c
-    const long long C = (long long)(((cb & kFrac52) | kHidden52) << 1);
-    const double x[6] = {x0, x1, x2, x3, x4, x5};
-    bool ok = true;
-    long long S = 0;
+__host__ __device__ __forceinline__ Lap6 lap6_units(double c, double x0, double x1, double x2, double x3, double x4,
+                                                    double x5) {
+    const unsigned long long b[7] = {dbits(x0), dbits(x1), dbits(x2), dbits(x3), dbits(x4), dbits(x5), dbits(c)};
+    unsigned h[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) h[i] = (unsigned)(b[i] >> 52);
+    const unsigned lo = umin3(umin3(h[0], h[1], h[2]), umin3(h[3], h[4], h[5]), h[6]);
+    const unsigned hi = umax3(umax3(h[0], h[1], h[2]), umax3(h[3], h[4], h[5]), h[6]);
+    Lap6 r;
+    r.h = lo;
+    const bool near = hi - lo <= 7u;  // exponents within 7, and one sign (else hi - lo >= 2^11 - 2046)
+    const long long C = significand(b[6], h[6] - lo);
+    unsigned acc = 0;
+    r.S = 0;
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
-        unsigned d;
-        const long long D = lap_units(x[i], hc, C, d) - C;
-        ok = ok && d <= 2u && (unsigned long long)(D + (1ll << 50)) < (1ull << 51);
-        S += D;
+        r.D[i] = significand(b[i], h[i] - lo) - C;
+        r.S += r.D[i];
+        acc |= mag_hi(r.D[i]) | mag_hi(r.S);
     }
-    return {S, ok && lap_c_ok(cb, S)};
+    // all +0: the hidden bits cancel, every difference is 0 (a positive subnormal's is positive, so S = 0 tells)
+    r.ok = near && (((lo & 0x7ffu) - 64u <= 1993u - 64u) || (b[6] == 0ull && r.S == 0));
+    r.exact = r.ok && acc < (1u << 21);
+    return r;
 }
 
-__host__ __device__ __forceinline__ bool lap6_exact_diffs(double c, double x0, double x1, double x2, double x3,
-                                                          double x4, double x5) {
-    const unsigned long long cb = dbits(c);
-    const unsigned hc = (unsigned)(cb >> 52);
-    const long long C = (long long)(((cb & kFrac52) | kHidden52) << 1);
-    const double x[6] = {x0, x1, x2, x3, x4, x5};
-    bool ok = true;
-    long long S = 0;
+// an integer rounded to 53 significant bits, to nearest even
+__host__ __device__ __forceinline__ long long round53(long long v) {
+    if (mag_hi(v) < (1u << 21)) return v;
+    const unsigned long long A = (unsigned long long)(v < 0 ? -v : v);
+    const int k = 11 - clz64(A);  // bits beyond 53 (A = 2^53 itself has one, and drops a zero)
+    const unsigned long long rem = A & ((1ull << k) - 1), half = 1ull << (k - 1);
+    unsigned long long q = A >> k;
+    q += (rem > half || (rem == half && (q & 1ull))) ? 1ull : 0ull;
+    const long long m = (long long)(q << k);
+    return v < 0 ? -m : m;
+}
+
+// L in units u with every operation rounded as the FP64 order rounds it (valid when ok)
+__host__ __device__ __forceinline__ long long lap6_rounded(const long long (&D)[6]) {
+    long long P = round53(round53(D[0]) + round53(D[1]));
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        unsigned d;
-        const long long X = lap_units(x[i], hc, C, d);
-        ok = ok && d <= 2u && 2 * X >= C && X <= 2 * C;
-        S += X - C;
-    }
-    return ok && lap_c_ok(cb, S);
+    for (int i = 2; i < 6; ++i) P = round53(P + round53(D[i]));
+    return P;
 }
 
-// S u with u = 2^(e_c - 1076), |S| < 2^54 with at most 53 significant bits: |S| = mant 2^-(lz - 11), mant in
-// [2^52, 2^53), biased exponent e_c + 10 - lz; the sign is c's times S's; 0 gives +0
-__host__ __device__ __forceinline__ double pack_units(long long S, double c) {
-    const unsigned long long cb = dbits(c);
-    const unsigned ec = (unsigned)(cb >> 52) & 0x7ffu;
+// S u with u = 2^(e - 1075), h the sign and biased exponent e; S has at most 53 significant bits and |S| < 2^63: with lz
+// leading zeros |S| 2^lz has its top bit at 63, so |S| = mant 2^(11 - lz) with mant = (|S| 2^lz) 2^-11 in [2^52, 2^53), and the
+// biased exponent is e + 11 - lz (mant's hidden bit adds the last 1); the sign is h's times S's; 0 gives +0
+__host__ __device__ __forceinline__ double pack_units(long long S, unsigned h) {
     const unsigned long long A = (unsigned long long)(S < 0 ? -S : S);
     const int lz = clz64(A);
-    const int sh = 11 - lz;
-    const unsigned long long mant = sh > 0 ? A >> sh : A << ((-sh) & 63);
-    const unsigned long long sign = (cb ^ (S < 0 ? (1ull << 63) : 0ull)) & (1ull << 63);
-    return A == 0 ? 0.0 : bits_d(sign | ((((unsigned long long)(ec + 10u - (unsigned)lz) - 1ull) << 52) + mant));
+    const unsigned long long mant = (A << (lz & 63)) >> 11;
+    const unsigned sign = ((h << 20) ^ (unsigned)((unsigned long long)S >> 32)) & 0x80000000u;
+    const unsigned long long top = (unsigned long long)(sign | (((h & 0x7ffu) + 10u - (unsigned)lz) << 20)) << 32;
+    return A == 0 ? 0.0 : bits_d(top + mant);
 }
 
-// x - c from integers (valid when the stencil passed exact_diffs)
-__host__ __device__ __forceinline__ double lap_diff(double x, double c) {
-    const unsigned long long cb = dbits(c);
-    unsigned d;
-    const long long C = (long long)(((cb & kFrac52) | kHidden52) << 1);
-    return pack_units(lap_units(x, (unsigned)(cb >> 52), C, d) - C, c);
-}
-
-// L from integers; false when some operation of the FP64 order might round (then L is not set)
+// L from integers; false when the stencil is left to FP64 (then L is not set)
 __host__ __device__ __forceinline__ bool lap6_int(double c, double x0, double x1, double x2, double x3, double x4,
                                                   double x5, double& L) {
-    const Lap6Sum k = lap6_exact_sum(c, x0, x1, x2, x3, x4, x5);
-    if (k.exact) L = pack_units(k.S, c);
-    return k.exact;
+    const Lap6 k = lap6_units(c, x0, x1, x2, x3, x4, x5);
+    if (k.ok) L = pack_units(k.exact ? k.S : lap6_rounded(k.D), k.h);
+    return k.ok;
 }
 
-// the six differences from integers, in one pass; false (d not set) unless every difference is exact
+// the six differences from integers; false (d not set) when the stencil is left to FP64
 __host__ __device__ __forceinline__ bool lap6_diffs(double c, double x0, double x1, double x2, double x3, double x4,
                                                     double x5, double (&d)[6]) {
-    const unsigned long long cb = dbits(c);
-    const unsigned hc = (unsigned)(cb >> 52);
-    const long long C = (long long)(((cb & kFrac52) | kHidden52) << 1);
-    const double x[6] = {x0, x1, x2, x3, x4, x5};
-    bool ok = true;
-    long long D[6], S = 0;
+    const Lap6 k = lap6_units(c, x0, x1, x2, x3, x4, x5);
+    if (k.ok) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        unsigned e;
-        const long long X = lap_units(x[i], hc, C, e);
-        ok = ok && e <= 2u && 2 * X >= C && X <= 2 * C;
-        D[i] = X - C;
-        S += D[i];
+        for (int i = 0; i < 6; ++i) d[i] = pack_units(round53(k.D[i]), k.h);
     }
-    ok = ok && lap_c_ok(cb, S);
-    if (ok) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) d[i] = pack_units(D[i], c);
-    }
-    return ok;
+    return k.ok;
 }
 
 // t = 2c - prev rounded once to nearest-even (the leapfrog's first operation), from integers where c is normal in the

@@ -109,7 +109,7 @@ int launch_sweep_f32k_tma(hg_grid* g, const SweepArgs& A) {
 }
 
 // the batched-launch entry of grid g for its sub-step cur -> 1 - cur: all ghosts inside the launch
-int tma_entry(hg_grid* g, TmaEntry* e, int zb) {
+int tma_entry(hg_grid* g, BatchEntry* e, int zb) {
     int rc = tma_maps(g);
     if (rc) return rc;
     const int c = g->cur;

@@ -1,5 +1,5 @@
 // Pieces of the compensated-float sub-step shared by the TMA-staged sweep (stencil_tma.cu, also the batched launch) and
-// the small-grid sweep (stencil_small.cu): a lane's 4-cell group update, its stores, and the periodic ghosts of the
+// the flat sweep (sweep_flat.cuh): a lane's 4-cell group update, its stores, and the periodic ghosts of the
 // new level.  Both sweeps thereby compute and store bit-identical results.
 #pragma once
 
@@ -61,8 +61,5 @@ __device__ __forceinline__ void group_update_store(const Layout& L, const Bnd& B
         });
     }
 }
-
-__device__ __forceinline__ int block_tid() { return threadIdx.y * blockDim.x + threadIdx.x; }
-__device__ __forceinline__ int block_nth() { return blockDim.x * blockDim.y; }
 
 }  // namespace hg

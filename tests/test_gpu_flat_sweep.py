@@ -1,9 +1,11 @@
-"""The small-grid sub-step (one thread per group of cells, all ghosts in one launch) against the z-marching sweeps, which a
-pinned block depth selects: the same arithmetic on the same values, so every cell and ghost must agree bit for bit,
-for rows shorter than a group, ragged rows, single rows and planes, every boundary condition and both precisions."""
+"""The flat sub-step (one thread per group of cells, all ghosts in one launch): float grids against the z-marching sweep,
+which a pinned block depth selects (the same arithmetic on the same values: every cell and ghost agrees bit for bit),
+FP64 grids against the oracle bit for bit, for rows shorter than a group, ragged rows, single rows and planes, and
+every boundary condition."""
 import numpy as np
 import pytest
 
+import oracle as O
 from paper_1602_05700_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -13,32 +15,54 @@ if not torch.cuda.is_available():  # pragma: no cover
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
 import paper_1602_05700_gb300 as hg  # noqa: E402
-from tests.test_gpu_parity import robin_cfl  # noqa: E402
+from tests.test_gpu_parity import BC_PAIRS, robin_cfl  # noqa: E402
 
 
-@pytest.mark.parametrize("shape", [(1, 1, 1), (3, 2, 1), (4, 1, 9), (5, 7, 3), (33, 17, 10), (129, 9, 6), (64, 64, 20)])
-@pytest.mark.parametrize("bc", ["dirichlet", "robin", "periodic"])
-@pytest.mark.parametrize("prec", ["f32k", "f64"])
-def test_small_grid_equals_marching_sweep(prec, bc, shape):
+SHAPES = [(1, 1, 1), (3, 2, 1), (4, 1, 9), (5, 7, 3), (33, 17, 10), (129, 9, 6), (64, 64, 20)]
+
+
+def case(shape, bc, prec):
     nx, ny, nz = shape
     h = 1.0 / 64
     dt = (robin_cfl(nx, ny, nz, h) if bc == "robin" else 0.5) * h / np.sqrt(3.0)
-    rho = I.noise(shape[::-1], 301, 0.0, 2.0)
+    origin = (-0.5 * nx * h, -0.5 * ny * h, -0.5 * nz * h)
     phi0 = I.noise(shape[::-1], 302, -1.0, -0.5)
     prev0 = phi0 + 1e-3 * I.noise(shape[::-1], 303, -1.0, 1.0)
+    g = hg.Grid(nx, ny, nz, h, origin, 1.0, 1.0, dt, prec, bc)
+    og = O.Grid(nx, ny, nz, h, origin, 1.0, 1.0, dt, BC_PAIRS[bc])
+    return g, og, I.noise(shape[::-1], 301, 0.0, 2.0), phi0, prev0
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("bc", ["dirichlet", "robin", "periodic"])
+def test_float_flat_equals_marching_sweep(bc, shape):
     out = []
     for depth in (0, 5):
-        g = hg.Grid(nx, ny, nz, h, (-0.5 * nx * h, -0.5 * ny * h, -0.5 * nz * h), 1.0, 1.0, dt, prec, bc)
+        g, _, rho, phi0, prev0 = case(shape, bc, "f32k")
         g.set_block_depth(depth)
         g.set_density(torch.from_numpy(rho).cuda())
         g.set_phi(torch.from_numpy(phi0).cuda(), torch.from_numpy(prev0).cuda())
-        g.step(9)
-        g.set_block_depth(depth)
-        g.step(2)
+        g.step(11)
         out.append((g.phi_ghosted(), g.stats()["change_rel"]))
         g.free()
     assert np.array_equal(out[0][0], out[1][0])
     assert out[0][1] == out[1][1]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("bc", ["dirichlet", "robin", "periodic"])
+def test_fp64_flat_equals_the_oracle(bc, shape):
+    """Bit for bit; without a density where it would bring in a sum (the periodic mean, the Dirichlet monopole)."""
+    g, og, rho, phi0, prev0 = case(shape, bc, "f64")
+    if bc != "robin":
+        rho = np.zeros_like(rho)
+    g.set_density(torch.from_numpy(rho).cuda())
+    g.set_phi(torch.from_numpy(phi0).cuda(), torch.from_numpy(prev0).cuda())
+    p, q = O.initial_state(og, rho, phi0=phi0, phi_prev0=prev0)
+    g.step(11)
+    O.run(og, p, q, rho, 11)
+    assert np.array_equal(g.phi(torch.float64, "cpu"), p[1:-1, 1:-1, 1:-1])
+    g.free()
 
 
 @pytest.mark.parametrize("prec", ["f32k", "f64"])
