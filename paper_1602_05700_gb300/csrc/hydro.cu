@@ -134,13 +134,30 @@ int ensure_hydro_staging(hg_hydro* H) {
     return HG_OK;
 }
 
-// z planes per block: about 1200 blocks in total (several waves of the 152 SMs), at least 8 planes per block
+// z planes per block.  FP32: about 2800 blocks, at least 8 planes each (280^3: 765 us per stage with 74 planes, 716 with
+// 32, 760 with 8).  FP64: the pipe of each SM is the bound, so the planes go out as evenly over the SMs as chunks of 6 to
+// 16 allow; a block's start-up is worth 0.9 planes (96^3: 12 planes, 288 blocks, 1782 us against 1845 with 8, 432 blocks;
+// 140^3: 14 planes 6059 against 6296 with 11; measured before the integer comparisons).
 int stage_zb(const hg_hydro* H) {
     const long long nxy = (long long)((H->nx + TX - 1) / TX) * ((H->ny + TY - 1) / TY);
-    long long zb = (H->nz * nxy + 1199) / 1200;
-    if (zb < 8) zb = 8;
+    long long zb = 0;
+    if (H->dtype == HG_DT_F64) {
+        double best = 0.0;
+        for (int z = 6; z <= 16; ++z) {
+            const long long blocks = nxy * ((H->nz + z - 1) / z);
+            const double cost = (double)((blocks + 151) / 152) * (z + 0.9);
+            if (!zb || cost < best) {
+                zb = z;
+                best = cost;
+            }
+        }
+    } else {
+        zb = (H->nz * nxy + 2799) / 2800;
+        if (zb < 8) zb = 8;
+    }
     if (zb > H->nz) zb = H->nz;
-    return (int)zb;
+    const long long chunks = (H->nz + zb - 1) / zb;  // even chunks
+    return (int)((H->nz + chunks - 1) / chunks);
 }
 
 constexpr int kHydroProfPairs = 1024;
