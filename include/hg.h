@@ -125,7 +125,7 @@ int hg_step(hg_grid* g, int n_substeps);
  * changed compensation can flip the rounding of a later increment), both staying within the compensated scheme's
  * accuracy against FP64.  With hg_set_temporal_exact(g, 1) the inner levels round their compensation as a store and a
  * load would, and the results are bit-identical to k single sweeps, at some cost in speed (measured at k = 2, 512^3,
- * Robin: 0.424 ms per sub-step by default, 0.519 exact, 0.503 for single sweeps).  k = 2 on Dirichlet and Robin grids
+ * Robin: 0.408 ms per sub-step by default, 0.476 exact, 0.505 for single sweeps).  k = 2 on Dirichlet and Robin grids
  * runs a TMA-staged kernel; other depths and periodic grids a generic one (slower than single sweeps).
  */
 #define HG_MAX_TEMPORAL_DEPTH 8

@@ -8,9 +8,9 @@
 //     writes it into a two-slot shared ring, then level n+2 of the same row one plane behind; warp 0 computes
 //     level n+1 of the two halo rows 0 and 9;
 //   * the helper warp (warp 9) issues the bulk-tensor copies of level n (plane by plane into a ring of 4 stages:
-//     hi and lo-code rows j0-2 .. j0+9, dlt and s rows j0-1 .. j0+8, all over cells x0-4 .. x0+131), computes
-//     level n+1 of the two halo columns x0-1 and x0+128 (20 single cells: no halo is recomputed by whole warps,
-//     so a 512-cell row takes exactly 4 tiles) and writes the level-(n+2) x-face ghosts.
+//     hi and lo-code rows j0-2 .. j0+9, dlt and s rows j0-1 .. j0+8, all over cells x0-4 .. x0+131), writes the
+//     level-(n+2) x-face ghosts and computes level n+1 of the two halo columns x0-1 and x0+128 (20 single cells: no halo
+//     is recomputed by whole warps, so a 512-cell row takes exactly 4 tiles).
 // In z the two levels form a pipeline: iteration `it` computes level n+1 at plane p = k0-1+it (own row's -z/centre
 // planes of level n in registers, +z and the y rows from the stages) and level n+2 at plane p-1 (own row's level
 // n+1 planes p-2, p-1, p in registers, the neighbouring rows and halo columns at p-1 from the ring); one block
@@ -23,6 +23,12 @@
 // (hg_set_temporal_exact) they go through the code as a store and a load would (lo_round4) and every cell update is
 // the single sweep's scalar form (cell.cuh), so the result is then bit-identical to two single sweeps; the default
 // mode runs the update on packed float pairs.
+//
+// Measured per sub-step (Robin, default mode, before -> after the two tile kinds were taken apart, the x-face coefficients
+// moved to shared memory and the first copies put before everything else a block does): 512^3 422 -> 408 us, 320^3 292 ->
+// 135, 200^3 90 -> 41, 301 x 259 x 223 182 -> 107; exact mode at 512^3 517 -> 476.
+// Tried without gain: the y-face rows' coefficients a plane ahead in registers (422 -> 429, spills), one rolled copy of the
+// level-(n+1) row for warp 0's two rows and the other warps (982: the shared state spills into the loop).
 //
 // HBM bytes per cell for the two sub-steps: 24 (read hi, lo, dlt, s; write hi, lo, dlt) plus the halo rows and
 // planes of neighbouring tiles (mostly served by L2).  Every wait is bounded in time; a wait that gives up sets the
@@ -53,7 +59,9 @@ struct F2 {
     static constexpr int stage = s_off + align128(d_tx);
     static constexpr int ring_off = kFS * stage;
     static constexpr int ring_slot = kFR * kFC;  // floats per slot (hi; the lo slots follow all hi slots)
-    static constexpr int smem = ring_off + 2 * 2 * ring_slot * 4;
+    static constexpr int coef_off = ring_off + 2 * 2 * ring_slot * 4;
+    static constexpr int planes = 32;  // most planes a block takes
+    static constexpr int smem = coef_off + 2 * planes * kFR * 8;
 };
 
 __device__ __forceinline__ float2 coef(const Bnd& B, int f, long long t) { return B.robin32[B.off[f] + t]; }
@@ -75,9 +83,13 @@ __device__ __forceinline__ void robin4(const Bnd& B, int f, long long t0, const 
     }
 }
 
-// One block: RAGGED is set for the last tile in x when nx is not a multiple of 128 (then the +x ghost lies inside
-// the tile and every lane classifies its cells); otherwise the x halo columns are the helper's.
-template <bool RAGGED, bool EXACT>
+// One block.  WHOLE: every tile is 128 cells wide -- nx >= 128 is a multiple of 8, and where it is not one of 128 the last tile
+// starts at nx - 128 and shares columns with its neighbour (both compute and store the same values; a bulk copy of the
+// 16-bit codes has to start on a multiple of 8 cells) -- so that the x halo columns are always the helper's.  Otherwise the
+// last tile may be ragged, with the +x ghost inside it, in one lane of each row warp; all tiles then run that more general
+// code: with a copy of each kind in one kernel the blocks that share an SM fetched more instructions than its cache holds
+// (52% of all stall cycles on a grid with ragged tiles).
+template <bool WHOLE, bool EXACT>
 __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUtensorMap* m_lo, const CUtensorMap* m_d,
                                              const CUtensorMap* m_s, const SweepArgs& A, float* __restrict__ d_out,
                                              int* err, unsigned char* smem, unsigned long long* bar_full,
@@ -86,7 +98,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     const Bnd& B = A.B;
     const bool robin = B.faces != 0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int x0 = blockIdx.x * kFX, j0 = blockIdx.y * kFY;
+    const int x0 = WHOLE ? min((int)blockIdx.x * kFX, L.nx - kFX) : (int)blockIdx.x * kFX, j0 = blockIdx.y * kFY;
     const int k0 = blockIdx.z * A.zb, k1 = min(L.nz, k0 + A.zb);
     const int nload = k1 - k0 + 3;  // level-n planes k0-1 .. k1+1: stage index i holds plane k0-1+i
     const int iters = k1 - k0 + 2;  // level n+1 at planes k0-1 .. k1
@@ -120,63 +132,42 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     auto Ss = [&](int i) { return (const float*)(stage_ptr(i) + F2::s_off); };
     auto rh = [&](int slot, int r, int col) { return ring_h + slot * F2::ring_slot + r * kFC + col; };
     auto rl = [&](int slot, int r, int col) { return ring_l + slot * F2::ring_slot + r * kFC + col; };
+    // Robin coefficients of the x-face ghosts of rows 0 .. 9 at the tile's planes, copied to shared memory once: a global
+    // load in the plane that uses it would hold up every plane of the block by an L2 latency, since all warps meet at
+    // its barrier
+    int issued = 0;  // the first copies go out before
+    if (warp == kFHelper && lane == 0)
+        for (; issued < kFS && issued < nload; ++issued) issue(issued);
+    float2* cx = (float2*)(smem + F2::coef_off);
+    if (robin)
+        for (int t = threadIdx.x; t < 2 * (k1 - k0) * kFR; t += kFThreads) {
+            const int f = t / ((k1 - k0) * kFR), u = t % ((k1 - k0) * kFR), y = j0 - 1 + u % kFR;
+            if (y >= 0 && y < L.ny && (f ? x0 + kFX >= L.nx : x0 == 0))
+                cx[t] = coef(B, f, (long long)(k0 + u / kFR) * L.ny + y);
+        }
+    auto xcoef = [&](int f, int pl, int r) { return cx[(f * (k1 - k0) + pl - k0) * kFR + r]; };  // k0 <= pl < k1
+    __syncthreads();
 
     if (warp == kFHelper) {
         // ---------------- helper: copies, level n+1 of the halo columns, level-(n+2) x-face ghosts ----------------
-        int issued = 0;
-        if (lane == 0)
-            for (; issued < kFS && issued < nload; ++issued) issue(issued);
         // lanes 0..9: column x0-1 of row r = lane; lanes 16..25: column x0+128 of row r = lane-16
         const int side = lane >> 4, r = lane & 15;
         const int col = side ? kFX + 4 : 3, xh = side ? x0 + kFX : x0 - 1;
         const int y = j0 - 1 + r;
-        const bool mine = r < kFR && y >= 0 && y < L.ny && (side ? (!RAGGED && xh <= L.nx) : true);
+        const bool mine = r < kFR && y >= 0 && y < L.ny && (side ? xh <= L.nx : true);
         const bool ghost = mine && (xh == -1 || xh == L.nx);  // an x-face ghost (only the tiles at the faces)
         const int sr = r + 1;
         float hm = 0.f, lm = 0.f;  // level n at plane p-1 of this lane's cell
+        const int ci = side ? col - 1 : col + 1;  // a ghost's interior neighbour
+        const int cj = side ? col + 1 : col - 1;
         for (int it = 0; it < iters; ++it) {
             const int p = k0 - 1 + it;
-            bool ok = it > 0 || wait_stage(0);
-            ok = ok && wait_stage(it + 1);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok && mine) {
-                const float* H = Hs(it);
-                const lo_t* Lo = Ls(it);
-                const float hc = H[sr * kFC + col], lc = lo_decode(hc, Lo[sr * kFC + col]);
-                if (p >= k0 && p < k1) {  // the ring needs the halo columns at the tile's own planes only
-                    float a = hc, b = lc;
-                    if (ghost) {
-                        if (robin) {
-                            const int ci = side ? col - 1 : col + 1;  // the interior neighbour
-                            const float hin = H[sr * kFC + ci];
-                            const float2 ab = coef(B, side, (long long)p * L.ny + y);
-                            robin_update_f32k(ab.x, ab.y, hc, lc, hin, lo_decode(hin, Lo[sr * kFC + ci]), a, b);
-                            if (EXACT) b = lo_round(a, b);
-                        }
-                    } else {
-                        const float* Hp = Hs(it + 1);
-                        const lo_t* Lp = Ls(it + 1);
-                        const float xl = H[sr * kFC + col - 1], xr = H[sr * kFC + col + 1];
-                        const float ys = H[(sr - 1) * kFC + col], yn = H[(sr + 1) * kFC + col];
-                        const float zp = Hp[sr * kFC + col];
-                        float c;
-                        f32k_update(xl, xr, ys, yn, hm, zp, hc, lo_decode(xl, Lo[sr * kFC + col - 1]),
-                                    lo_decode(xr, Lo[sr * kFC + col + 1]), lo_decode(ys, Lo[(sr - 1) * kFC + col]),
-                                    lo_decode(yn, Lo[(sr + 1) * kFC + col]), lm, lo_decode(zp, Lp[sr * kFC + col]), lc,
-                                    Ds(it)[r * kFC + col], Ss(it)[r * kFC + col], nu2, a, b, c);
-                        if (EXACT) b = lo_round(a, b);
-                    }
-                    *rh(it & 1, r, col) = a;
-                    *rl(it & 1, r, col) = b;
-                }
-                hm = hc;
-                lm = lc;
-            }
-            // level-(n+2) x-face ghosts at plane q = p-1 (Robin), rows 1..8, from the ring written last iteration
+            // level-(n+2) x-face ghosts at plane q = p-1 (Robin), rows 1..8, from the ring written last iteration (before
+            // the waits: this warp's chain must not be the plane's longest)
             const int q = p - 1;
-            if (ok && ghost && robin && r >= 1 && r <= kFY && q >= k0 && q < k1) {
-                const int slot = (it - 1) & 1, ci = side ? col - 1 : col + 1;
-                const float2 ab = coef(B, side, (long long)q * L.ny + y);
+            if (ghost && robin && r >= 1 && r <= kFY && q >= k0 && q < k1 && !*abort_flag) {
+                const int slot = (it - 1) & 1;
+                const float2 ab = xcoef(side, q, r);
                 float a, b;
                 robin_update_f32k(ab.x, ab.y, *rh(slot, r, col), *rl(slot, r, col), *rh(slot, r, ci),
                                   *rl(slot, r, ci), a, b);
@@ -185,6 +176,38 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
                     hi_n[qi] = a;
                     lo_n[qi] = lo_encode(a, b);
                 }
+            }
+            bool ok = it > 0 || wait_stage(0);
+            ok = ok && wait_stage(it + 1);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && mine) {
+                const float* H = Hs(it);
+                const lo_t* Lo = Ls(it);
+                const float hc = H[sr * kFC + col], lc = lo_decode(hc, Lo[sr * kFC + col]);
+                if (p >= k0 && p < k1) {  // the ring needs the halo columns at the tile's own planes only
+                    // the stencil and, for an x-face ghost, its own rule, without a branch between them (a warp whose two
+                    // halves differ would run one after the other)
+                    const float* Hp = Hs(it + 1);
+                    const lo_t* Lp = Ls(it + 1);
+                    const float xi = H[sr * kFC + ci], xj = H[sr * kFC + cj];
+                    const float li = lo_decode(xi, Lo[sr * kFC + ci]), lj = lo_decode(xj, Lo[sr * kFC + cj]);
+                    const float ys = H[(sr - 1) * kFC + col], yn = H[(sr + 1) * kFC + col];
+                    const float zp = Hp[sr * kFC + col];
+                    const float2 ab = robin && ghost ? xcoef(side, p, r) : make_float2(1.f, 0.f);
+                    float a, b, c, ag, bg;
+                    robin_update_f32k(ab.x, ab.y, hc, lc, xi, li, ag, bg);
+                    f32k_update(side ? xi : xj, side ? xj : xi, ys, yn, hm, zp, hc, side ? li : lj, side ? lj : li,
+                                lo_decode(ys, Lo[(sr - 1) * kFC + col]), lo_decode(yn, Lo[(sr + 1) * kFC + col]), lm,
+                                lo_decode(zp, Lp[sr * kFC + col]), lc, Ds(it)[r * kFC + col], Ss(it)[r * kFC + col],
+                                nu2, a, b, c);
+                    a = ghost ? (robin ? ag : hc) : a;
+                    b = ghost ? (robin ? bg : lc) : b;
+                    if (EXACT && (robin || !ghost)) b = lo_round(a, b);
+                    *rh(it & 1, r, col) = a;
+                    *rl(it & 1, r, col) = b;
+                }
+                hm = hc;
+                lm = lc;
             }
             __syncthreads();
             if (lane == 0 && !*abort_flag && it + kFS < nload) {  // every warp is done with plane p's stage
@@ -205,12 +228,27 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     // halo rows 0 and 9 (y = j0-1 and j0+8), and the level-(n+2) y-face ghost row when one of them is a ghost row
     const int xa = x0 + 4 * lane;  // first cell of this lane's group
     const int col = 4 + 4 * lane;  // its stage / ring column
-    // RAGGED tiles: the class of each of the lane's cells in x -- 0 interior, 2 the +x ghost, 3 beyond it
-    int xc[4] = {0, 0, 0, 0};
-    if (RAGGED)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) xc[e] = xa + e < L.nx ? 0 : xa + e == L.nx ? 2 : 3;
-    const int nlive = RAGGED ? max(0, min(4, L.nx - xa)) : 4;  // interior cells of the group
+    const int nlive = WHOLE ? 4 : max(0, min(4, L.nx - xa));  // interior cells of the group
+    // the element of the group that is the +x ghost, or -1 (in a ragged tile one lane of each row warp has it)
+    const int ge = !WHOLE && L.nx >= xa && L.nx < xa + 4 ? L.nx - xa : -1;
+    // the ghost's value of the next level from the group's values (h, l) and the cell before the group (xl, ll): unchanged
+    // (Dirichlet, or a plane beyond the tile, where nothing uses it) or its Robin update
+    auto ghost_update = [&](const float4& h, const float4& l, float xl, float ll, int pl, int r, float& a, float& b) {
+        a = ge == 0 ? h.x : ge == 1 ? h.y : ge == 2 ? h.z : h.w;
+        b = ge == 0 ? l.x : ge == 1 ? l.y : ge == 2 ? l.z : l.w;
+        const float hi = ge == 0 ? xl : ge == 1 ? h.x : ge == 2 ? h.y : h.z;
+        const float li = ge == 0 ? ll : ge == 1 ? l.x : ge == 2 ? l.y : l.z;
+        if (robin && pl >= k0 && pl < k1) {
+            const float2 ab = xcoef(1, pl, r);
+            robin_update_f32k(ab.x, ab.y, a, b, hi, li, a, b);
+        }
+    };
+    auto put = [&](float4& v, float x) {  // v's element ge
+        v.x = ge == 0 ? x : v.x;
+        v.y = ge == 1 ? x : v.y;
+        v.z = ge == 2 ? x : v.z;
+        v.w = ge == 3 ? x : v.w;
+    };
 
     struct Row {
         int r, y, sr;
@@ -240,7 +278,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
         l1 = lc0;
         d1 = d0;
         if (R.in && p >= 0 && p < L.nz) {
-            // interior plane of an interior row: the stencil (RAGGED: the +x ghost cell by its boundary rule)
+            // interior plane of an interior row: the stencil (the +x ghost cell by its boundary rule)
             const float* Hp = Hs(it + 1);
             const float4 hp0 = lds4(Hp + sr * kFC + col);
             const float4 lp0 = lo_decode4(hp0, ldsl4(Ls(it + 1) + sr * kFC + col));
@@ -262,21 +300,12 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
             else
                 f32k_update4(hc0, lc0, hl, ll, hr, lr, hs, hn, hm0, hp0, ls, ln, lm0, lp0, d0, s0, nu2, h1, l1, d1);
             if (EXACT) l1 = lo_round4(h1, l1);
-            if (RAGGED) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (xc[e] == 2) {  // the +x ghost: keeps level n (Dirichlet) or its Robin update
-                        float a = el(hc0, e), b = el(lc0, e);
-                        if (robin) {
-                            const float2 ab = coef(B, 1, (long long)p * L.ny + y);
-                            const float gi = e == 0 ? hl : el(hc0, e - 1), li = e == 0 ? ll : el(lc0, e - 1);
-                            robin_update_f32k(ab.x, ab.y, el(hc0, e), el(lc0, e), gi, li, a, b);
-                            if (EXACT) b = lo_round(a, b);
-                        }
-                        set(h1, e, a);
-                        set(l1, e, b);
-                        set(d1, e, el(d0, e));
-                    }
+            if (!WHOLE && ge >= 0) {
+                float a, b;
+                ghost_update(hc0, lc0, hl, ll, p, r, a, b);
+                if (EXACT && robin) b = lo_round(a, b);
+                put(h1, a);
+                put(l1, b);
             }
         } else if (robin && R.in) {
             // a z-face ghost plane (p = -1 or nz) of an interior row: the radiation update
@@ -404,25 +433,23 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
                     f32k_update4(c1, lc1, gl, gll, gr, grl, ys, yn, m1, h1, lys, lyn, lm1, l1, d1c, sc, nu2, ho, lo, dout);
                 const long long qo = L.at(xa, y, q);
                 if (!idx_ok(qo, 4, L.elems, B.err)) {
-                } else if (!RAGGED || xa + 3 < L.nx) {
+                } else if (WHOLE || nlive == 4) {
                     *reinterpret_cast<float4*>(hi_n + qo) = ho;
                     *reinterpret_cast<uint2*>(lo_n + qo) = lo_encode4(ho, lo);
                     *reinterpret_cast<float4*>(d_out + qo) = dout;
                 } else {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        if (xc[e] == 0) {
+                    for (int e = 0; e < 4; ++e)
+                        if (e < nlive) {
                             hi_n[qo + e] = el(ho, e);
                             lo_n[qo + e] = lo_encode(el(ho, e), el(lo, e));
                             d_out[qo + e] = el(dout, e);
-                        } else if (xc[e] == 2 && robin) {  // the level-(n+2) +x ghost
-                            const float2 ab = coef(B, 1, (long long)q * L.ny + y);
-                            const float gi = e == 0 ? gl : el(c1, e - 1), li = e == 0 ? gll : el(lc1, e - 1);
-                            float a, b;
-                            robin_update_f32k(ab.x, ab.y, el(c1, e), el(lc1, e), gi, li, a, b);
-                            hi_n[qo + e] = a;
-                            lo_n[qo + e] = lo_encode(a, b);
                         }
+                    if (ge >= 0 && robin) {  // the level-(n+2) +x ghost
+                        float a, b;
+                        ghost_update(c1, lc1, gl, gll, q, r, a, b);
+                        hi_n[qo + ge] = a;
+                        lo_n[qo + ge] = lo_encode(a, b);
                     }
                 }
             } else if (robin && R.ghost && q >= k0 && q < k1) {
@@ -457,6 +484,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     }
 }
 
+template <bool WHOLE, bool EXACT>
 __global__ void __maxnreg__(96)  // 2 blocks of 320 threads per SM (5 warps of 96 registers per SM quarter)
     k_temporal2_tma(const __grid_constant__ CUtensorMap m_hi, const __grid_constant__ CUtensorMap m_lo,
                     const __grid_constant__ CUtensorMap m_d, const __grid_constant__ CUtensorMap m_s,
@@ -473,21 +501,10 @@ __global__ void __maxnreg__(96)  // 2 blocks of 320 threads per SM (5 warps of 9
     __syncthreads();
     pdl_trigger();
     pdl_wait();
-    const bool ragged = (int)(blockIdx.x * kFX) + kFX > A.L.nx;
-    if (A.exact) {
-        if (ragged)
-            fused2_block<true, true>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
-        else
-            fused2_block<false, true>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
-    } else {
-        if (ragged)
-            fused2_block<true, false>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
-        else
-            fused2_block<false, false>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
-    }
+    fused2_block<WHOLE, EXACT>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
 }
 
-constexpr int kZ2 = 32;  // level-(n+2) planes per block
+constexpr int kZ2 = F2::planes;  // level-(n+2) planes per block
 
 // tensor maps of the staged level-n state with this kernel's boxes: hi[0..1], lo[0..1], dlt[0..1], s
 int tma2_maps(hg_grid* g) {
@@ -512,16 +529,26 @@ int launch_temporal2_tma(hg_grid* g) {
         return fail(HG_ERR_STATE, "the TMA-staged depth-2 kernel needs a Dirichlet or Robin f32k grid with two dlt buffers");
     int rc = tma2_maps(g);
     if (rc) return rc;
-    static unsigned long long attr_done = 0;
-    if ((rc = smem_attr_once((const void*)k_temporal2_tma, F2::smem, &attr_done))) return rc;
-    const int zb = g->zb > 0 ? (g->zb < g->nz ? g->zb : g->nz) : (g->nz < kZ2 ? g->nz : kZ2);
+    const int zb0 = g->zb > 0 && g->zb < kZ2 ? g->zb : kZ2, zb = g->nz < zb0 ? g->nz : zb0;
     SweepArgs A = sweep_args(g, zb);
     A.B.faces = g->bc == HG_BC_ROBIN ? 1 : 0;
     A.B.periodic = 0;
     const int c = g->cur;
     dim3 grid((g->nx + kFX - 1) / kFX, (g->ny + kFY - 1) / kFY, (g->nz + zb - 1) / zb);
+    // which code (see fused2_block).  Whole tiles where nx allows them (320^3 139 against 173 us per sub-step, 512^3 422
+    // against 471 before the copies went first), except in exact mode on grids of more than one wave of blocks, where the general code comes out
+    // faster (512^3: 483 against 521 us; the register allocation of the scalar update differs), not on smaller ones
+    // (128^3: 32 against 37)
+    const bool whole = g->nx >= kFX && g->nx % 8 == 0;
+    const int v = g->texact ? (whole && (long long)grid.x * grid.y * grid.z <= 304 ? 0 : 1) : whole ? 2 : 3;
+    static unsigned long long attr_done[4] = {0, 0, 0, 0};
+    const auto kernel = v == 0   ? k_temporal2_tma<true, true>
+                        : v == 1 ? k_temporal2_tma<false, true>
+                        : v == 2 ? k_temporal2_tma<true, false>
+                                 : k_temporal2_tma<false, false>;
+    if ((rc = smem_attr_once((const void*)kernel, F2::smem, &attr_done[v]))) return rc;
     if ((rc = prof_begin(g))) return rc;
-    if ((rc = launch_pdl(k_temporal2_tma, grid, dim3(kFThreads), F2::smem, g->stream, g->tm2[0 + c], g->tm2[2 + c],
+    if ((rc = launch_pdl(kernel, grid, dim3(kFThreads), F2::smem, g->stream, g->tm2[0 + c], g->tm2[2 + c],
                          g->tm2[4 + g->dcur], g->tm2[6], A, (float*)g->dlt[1 - g->dcur], g->derr)))
         return rc;
     HG_LAUNCHED("TMA-staged depth-2 sub-step kernel");
