@@ -1,7 +1,12 @@
 // TMA-staged single sweep of the compensated-float sub-step (arXiv 1602.05700, Sec. 1 Eq. HNeq., Sec. 2): the
-// kernel of a single grid's sub-step (the sweep itself is tma_sweep in sweep_tma.cuh), and the host side of the
+// kernel of a large grid's sub-step (the sweep itself is tma_sweep in sweep_tma.cuh), and the host side of the
 // staging -- the 3-D tensor maps of a grid's state, built once through the driver's cuTensorMapEncodeTiled, and the
 // entries of the batched launch.
+//
+// Robin, us per sub-step, with a block's first copies sent before it meets and the producer's face ghosts taken out of the
+// way of its next copy (before -> after; floor at the copy bandwidth): 512^3 505 -> 497 (475), 320^3 148 -> 142 (116),
+// 301 x 259 x 223 87.7 -> 83.1 (62), 256^3 79.7 -> 77.7 (59).  What remains of the middle sizes is the last wave of blocks
+// (256^3: 2048 blocks on 456 places) and the z halo of 8-plane chunks.
 #include <cuda.h>
 
 #include "sweep_tma.cuh"

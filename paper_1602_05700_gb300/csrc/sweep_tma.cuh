@@ -124,28 +124,45 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
     const bool fy0 = B.faces && by == 0, fy1 = B.faces && by == (int)A.gy - 1;
     const bool faces = fx0 || fx1 || fy0 || fy1;
 
-    if (tid == 0) {
+    // the producer's issuing thread sets up the barriers and sends the first copies before the block meets (a block of 8
+    // planes is short: what it does before its first copy is paid every 14 us)
+    auto issue = [&](int it) {
+        const int s = it % S, p = k0 + it;
+        const uint32_t full = smem_addr(&bar_full[s]);
+        unsigned char* st = smem + s * G::bytes;
+        const bool body = p < k1;
+        mbar_expect_tx(full, G::h_tx + G::l_tx + (body ? 2 * G::d_tx : 0));
+        tma_load_3d(smem_addr(st + G::h_off), m_hi, x0, j0, p + 1, full);
+        tma_load_3d(smem_addr(st + G::l_off), m_lo, x0, j0, p + 1, full);
+        if (body) {
+            tma_load_3d(smem_addr(st + G::d_off), m_d, x0 + 4, j0 + 1, p + 1, full);
+            tma_load_3d(smem_addr(st + G::r_off), m_s, x0 + 4, j0 + 1, p + 1, full);
+        }
+    };
+    const int first = planes < S ? planes : S;
+    if (tid == 32 * WY) {
         for (int s = 0; s < S; ++s) {
             mbar_init(smem_addr(&bar_full[s]), 1);
             mbar_init(smem_addr(&bar_empty[s]), WY + (faces ? 1 : 0));
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        pdl_wait();  // single-grid launches start before the previous sub-step has ended; no effect in other launches
+        for (int it = 0; it < first; ++it) issue(it);
     }
     __syncthreads();
-    pdl_wait();  // single-grid launches start before the previous sub-step has ended; no effect in other launches
+    pdl_wait();
 
     if (warp == WY) {  // producer
-        constexpr int lag = S - 1;  // face work trails the copies by this many planes
         float* hi_n = (float*)A.hi_n;
         lo_t* lo_n = (lo_t*)A.lo_n;
         // face-ghost lanes: x faces -- lanes 0..WY-1 the rows of face -x, lanes 16..16+WY-1 those of face +x;
         // y faces -- every lane 4 ghosts of row -1 (first row of tiles) and/or row ny (last row of tiles)
         const int w = lane & 15, side = lane >> 4, jx = j0 + w;
         const bool xlane = w < WY && jx < L.ny && (side ? fx1 : fx0);
-        // Robin coefficients: the x-face ones travel to shared memory by asynchronous copies issued with each plane's
-        // bulk copies (`lag` planes before they are used, so their latency never reaches this warp); the y-face ones
-        // (first and last row of tiles only) are loaded one face plane ahead into registers
+        // Robin coefficients: the x-face ones travel to shared memory by asynchronous copies S - 1 planes before they are
+        // used, so their latency never reaches this warp; the y-face ones (first and last row of tiles only) are loaded one
+        // plane ahead into registers
         __shared__ float2 cxs[S][32];
         float2 cy[2][4];
         auto load_coef = [&](int k) {
@@ -158,49 +175,34 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
                                                               : make_float2(0.f, 0.f);
                 }
         };
-        if (faces) load_coef(k0);
-        int issued = 0;
+        auto copy_coef = [&](int n) {  // one copy group per plane (empty when there is nothing to copy)
+            if (xlane && n < planes - 1)
+                __pipeline_memcpy_async(&cxs[n % S][lane], &B.robin32[B.off[side] + (long long)(k0 + n) * L.ny + jx],
+                                        sizeof(float2));
+            __pipeline_commit();
+        };
+        if (faces) {
+            for (int n = 0; n < S - 1; ++n) copy_coef(n);
+            load_coef(k0);
+        }
+        int issued = first;
         bool ok = true;
-        for (int it = 0; it < planes + (faces ? lag : 0) && ok; ++it) {
-            if (it < planes) {
-                if (lane == 0) {
-                    const int s = it % S, p = k0 + it;
-                    if (it >= S) ok = mbar_wait(smem_addr(&bar_empty[s]), (unsigned)((it / S - 1) & 1), err);
-                    if (ok) {
-                        const uint32_t full = smem_addr(&bar_full[s]);
-                        unsigned char* st = smem + s * G::bytes;
-                        const bool body = p < k1;
-                        mbar_expect_tx(full, G::h_tx + G::l_tx + (body ? 2 * G::d_tx : 0));
-                        tma_load_3d(smem_addr(st + G::h_off), m_hi, x0, j0, p + 1, full);
-                        tma_load_3d(smem_addr(st + G::l_off), m_lo, x0, j0, p + 1, full);
-                        if (body) {
-                            tma_load_3d(smem_addr(st + G::d_off), m_d, x0 + 4, j0 + 1, p + 1, full);
-                            tma_load_3d(smem_addr(st + G::r_off), m_s, x0 + 4, j0 + 1, p + 1, full);
-                        }
-                        issued = it + 1;
-                    }
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                issued = __shfl_sync(0xffffffffu, issued, 0);
-            }
-            if (faces) {  // one copy group per iteration (empty when there is nothing to copy), so counts stay uniform
-                if (xlane && it < planes - 1)
-                    __pipeline_memcpy_async(&cxs[it % S][lane], &B.robin32[B.off[side] + (long long)(k0 + it) * L.ny + jx],
-                                            sizeof(float2));
-                __pipeline_commit();
-            }
-            const int pf = it - lag;  // plane (chunk-relative) whose face ghosts are due; the chunk's own planes only
-            if (faces && ok && pf >= 0 && pf < planes - 1) {
-                const int s = pf % S, k = k0 + pf;
-                __pipeline_wait_prior(lag);  // the copy group of plane pf has landed
+        // plane n of the chunk: its face ghosts while the consumers work on it, then, once they have released it, the next
+        // copy into its stage: the face work never stands between the release and the copy
+        for (int n = 0; n < planes - 1 && ok; ++n) {
+            const int s = n % S;
+            if (faces) {
+                const int k = k0 + n;
+                copy_coef(n + S - 1);
+                __pipeline_wait_prior(S - 1);  // the copy group of plane n has landed
                 const float2 ax = cxs[s][lane];
                 float2 ay[2][4];
 #pragma unroll
                 for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
                     for (int e = 0; e < 4; ++e) ay[s2][e] = cy[s2][e];
-                if (pf + 1 < planes - 1) load_coef(k + 1);
-                if (!(ok = mbar_wait(smem_addr(&bar_full[s]), (unsigned)((pf / S) & 1), err))) break;
+                if (n + 1 < planes - 1) load_coef(k + 1);
+                if (!(ok = mbar_wait(smem_addr(&bar_full[s]), (unsigned)((n / S) & 1), err))) break;
                 const float* H = (const float*)(smem + s * G::bytes + G::h_off);
                 const lo_t* Lo = (const lo_t*)(smem + s * G::bytes + G::l_off);
                 if (xlane) {
@@ -239,6 +241,17 @@ __device__ __forceinline__ void tma_sweep(const CUtensorMap* m_hi, const CUtenso
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_addr(&bar_empty[s]));
+            }
+            if (n + S < planes) {
+                if (lane == 0) {
+                    ok = mbar_wait(smem_addr(&bar_empty[s]), (unsigned)((n / S) & 1), err);
+                    if (ok) {
+                        issue(n + S);
+                        issued = n + S + 1;
+                    }
+                }
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                issued = __shfl_sync(0xffffffffu, issued, 0);
             }
         }
         // the copies still in flight belong to the last S issued stages; make sure they have landed before the block
