@@ -104,7 +104,7 @@ int upload_tables(hg_batch* b) {
                 rc = tma_entry(g, &e, b->zb32);
             } else {
                 e.A = sweep_args(g, 0);
-                e.G = flat_grid(g, kBatchThreads);
+                e.G = flat_grid(g, kBatchThreads, g->prec == HG_PREC_F32K ? 4 : 1);
                 e.err = g->derr;
             }
             g->cur = cur;

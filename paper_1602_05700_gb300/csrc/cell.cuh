@@ -180,6 +180,14 @@ __device__ __forceinline__ double lap6_fp64(double xl, double xr, double ys, dou
     return __dadd_rn(L, __dsub_rn(zp, c));
 }
 
+// An FP64 operation of one side of a branch: as a volatile instruction it stays there.  (The compiler evaluates a plain
+// expression on both sides and selects, which costs the warp the FP64 cycles that the branch is to save.)
+__device__ __forceinline__ double fma_here(double a, double b, double c) {
+    double r;
+    asm volatile("fma.rn.f64 %0, %1, %2, %3;" : "=d"(r) : "d"(a), "d"(b), "d"(c));
+    return r;
+}
+
 // The form is chosen per warp (the cheapest form every lane of the warp can take), so that a warp never executes two forms
 // one after the other: an FP64 instruction costs a warp 16 cycles of the SM's FP64 pipe whatever its active mask.  Each
 // form gives every lane the same bits.  2c - prev is an FP64 operation where L comes from integers (the integer pipes are
@@ -197,9 +205,34 @@ __device__ __forceinline__ double f64_update(double xl, double xr, double ys, do
     } else {
         L = lap6_fp64(xl, xr, ys, yn, zm, zp, c);
         const bool ti = twice_minus_int(c, prev, t);
-        if (!__all_sync(m, ti)) t = __fma_rn(2.0, c, -prev);
+        if (!__all_sync(m, ti)) t = fma_here(2.0, c, -prev);
     }
     return __dsub_rn(__dadd_rn(t, __dmul_rn(nu2, L)), s);
+}
+
+// The same for two cells of a lane next to each other along x (v[q]: the neighbours of cell q in the order of the sum)
+__device__ __forceinline__ void f64_update2(const double (&c)[2], const double (&v)[2][6], const double (&prev)[2],
+                                            const double (&s)[2], double nu2, double (&out)[2]) {
+    const unsigned m = __activemask();
+    const Lap6Pair k = lap6_units2(c, v);
+    double L[2], t[2];
+    if (__all_sync(m, k.ok)) {
+        const bool exact = __all_sync(m, k.exact);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            t[q] = __fma_rn(2.0, c[q], -prev[q]);
+            L[q] = pack_units(exact ? k.S[q] : lap6_rounded(k.D[q]), k.h);
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            L[q] = lap6_fp64(v[q][0], v[q][1], v[q][2], v[q][3], v[q][4], v[q][5], c[q]);
+            const bool ti = twice_minus_int(c[q], prev[q], t[q]);
+            if (!__all_sync(m, ti)) t[q] = fma_here(2.0, c[q], -prev[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) out[q] = __dsub_rn(__dadd_rn(t[q], __dmul_rn(nu2, L[q])), s[q]);
 }
 
 // Robin ghost sub-step in FP64 (monopole radiation condition, upwinded) for u = r phi:

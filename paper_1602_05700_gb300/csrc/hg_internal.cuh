@@ -333,7 +333,7 @@ struct FlatGrid {
     FastDiv per_plane, gpr;       // tiles per plane, groups per row
     int wide;                     // a plane holds 2^31 groups or more
 };
-FlatGrid flat_grid(const hg_grid* g, int threads);
+FlatGrid flat_grid(const hg_grid* g, int threads, int width);  // width: cells per group
 
 // a 3-D TMA map over a padded array (pitch x (ny+2) x (nz+2) elements of `bytes` each), boxes box_x x box_y x 1
 int tma_encode(CUtensorMap* m, void* base, const Layout& L, int bytes, int box_x, int box_y);

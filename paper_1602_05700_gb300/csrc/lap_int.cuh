@@ -129,6 +129,54 @@ __host__ __device__ __forceinline__ Lap6 lap6_units(double c, double x0, double 
     return r;
 }
 
+// Two cells next to each other along x in common units (the smallest ulp of their twelve values): the conversions of c0, c1
+// and their difference serve both.  v[q]: the neighbours of cell q in the order of the sum (v[0][1] is c1, v[1][0] is c0).
+struct Lap6Pair {
+    long long D[2][6];
+    long long S[2];
+    unsigned h;
+    bool exact, ok;
+};
+__host__ __device__ __forceinline__ Lap6Pair lap6_units2(const double (&c)[2], const double (&v)[2][6]) {
+    const unsigned long long b[12] = {dbits(c[0]),    dbits(c[1]),    dbits(v[0][0]), dbits(v[1][1]),
+                                      dbits(v[0][2]), dbits(v[0][3]), dbits(v[0][4]), dbits(v[0][5]),
+                                      dbits(v[1][2]), dbits(v[1][3]), dbits(v[1][4]), dbits(v[1][5])};
+    unsigned h[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) h[i] = (unsigned)(b[i] >> 52);
+    const unsigned lo = umin3(umin3(umin3(h[0], h[1], h[2]), umin3(h[3], h[4], h[5]), umin3(h[6], h[7], h[8])),
+                              umin3(h[9], h[10], h[11]), h[0]);
+    const unsigned hi = umax3(umax3(umax3(h[0], h[1], h[2]), umax3(h[3], h[4], h[5]), umax3(h[6], h[7], h[8])),
+                              umax3(h[9], h[10], h[11]), h[0]);
+    Lap6Pair r;
+    r.h = lo;
+    const bool near = hi - lo <= 7u;
+    long long m[12];
+#pragma unroll
+    for (int i = 0; i < 12; ++i) m[i] = significand(b[i], h[i] - lo);
+    const long long D01 = m[1] - m[0];
+    r.D[0][0] = m[2] - m[0];
+    r.D[0][1] = D01;
+    r.D[1][0] = -D01;
+    r.D[1][1] = m[3] - m[1];
+    unsigned acc = 0;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) r.D[q][2 + i] = m[4 + 4 * q + i] - m[q];
+        r.S[q] = 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            r.S[q] += r.D[q][i];
+            acc |= mag_hi(r.D[q][i]) | mag_hi(r.S[q]);
+        }
+    }
+    // all +0 as in lap6_units: with c0 = c1 = +0 no difference is negative
+    r.ok = near && (((lo & 0x7ffu) - 64u <= 1993u - 64u) || ((b[0] | b[1]) == 0ull && r.S[0] == 0 && r.S[1] == 0));
+    r.exact = r.ok && acc < (1u << 21);
+    return r;
+}
+
 // an integer rounded to 53 significant bits, to nearest even
 __host__ __device__ __forceinline__ long long round53(long long v) {
     if (mag_hi(v) < (1u << 21)) return v;

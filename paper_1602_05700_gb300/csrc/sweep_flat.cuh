@@ -98,4 +98,40 @@ __device__ __forceinline__ void flat_f64(const SweepArgs& A, int i, int j, int k
     }
 }
 
+// Two cells i, i+1 of an FP64 grid's row; `two` is false for the last cell of an odd row, whose partner is the +x ghost
+__device__ __forceinline__ void flat_f64x2(const SweepArgs& A, int i, int j, int k) {
+    const Layout& L = A.L;
+    const bool two = i + 1 < L.nx;
+    const long long q = L.at(i, j, k);
+    const double* p = (const double*)A.hi_c + q;
+    double* o = (double*)A.hi_n;
+    auto d2 = [](const double* a) { return *reinterpret_cast<const double2*>(a); };  // rows start on 128 bytes, i is even
+    const double2 cc = d2(p), ys = d2(p - L.pitch), yn = d2(p + L.pitch), zm = d2(p - L.plane), zp = d2(p + L.plane);
+    const double2 pv = d2(o + q), rs = d2((const double*)A.rho + q);
+    const double xl = p[-1], xr = p[two ? 2 : 1];
+    double n[2][6] = {{xl, cc.y, ys.x, yn.x, zm.x, zp.x}, {cc.x, xr, ys.y, yn.y, zm.y, zp.y}};
+    if (!two) {  // neighbours that leave the form of the first cell's sum as it is
+#pragma unroll
+        for (int e = 1; e < 6; ++e) n[1][e] = cc.y;
+    }
+    double v[2];
+    f64_update2({cc.x, cc.y}, n, {pv.x, pv.y}, {rs.x, rs.y}, A.nu2, v);
+    if (!idx_ok(q, 2, L.elems, A.B.err)) return;
+    if (two)
+        *reinterpret_cast<double2*>(o + q) = make_double2(v[0], v[1]);
+    else
+        o[q] = v[0];
+    if (A.B.periodic) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            if (e == 1 && !two) break;
+            auto put = [&](long long gq) {
+                if (idx_ok(gq, 1, L.elems, A.B.err)) o[gq] = v[e];
+            };
+            periodic_x_ghosts(L, i + e, q + e, put);
+            periodic_yz_ghosts(L, j, k, q + e, put);
+        }
+    }
+}
+
 }  // namespace hg
