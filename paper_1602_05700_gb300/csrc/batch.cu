@@ -9,8 +9,8 @@
 // Results are identical to stepping each grid on its own: the per-cell arithmetic is the same code.
 //
 // 48 grids of 64^3 to 192^3, alternating precisions, per sub-step: 2.18 ms with marching FP64 blocks and TMA-staged float
-// blocks in one launch (the FP64 half latency-bound at 16 warps per SM, 60% of a 96-cell row's tile in use), see
-// sweep_flat.cuh for what the flat sweep changes.
+// blocks in one launch (the FP64 half latency-bound at 16 warps per SM, 60% of a 96-cell row's tile in use), 1.05 with
+// the flat sweep (sweep_flat.cuh says what it changes).
 //
 // Autotuning: two knobs of the launch are chosen by timing the first sub-steps of the first hg_batch_step with CUDA
 // events -- every candidate computes the same result, so the timing runs are real sub-steps -- and cached per

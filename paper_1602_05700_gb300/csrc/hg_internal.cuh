@@ -171,7 +171,7 @@ struct hg_grid {
     int tdepth;
     int texact;  // fused sub-steps bit-identical to single sweeps (hg_set_temporal_exact)
     int ziface;  // bit 0 / bit 1: -z / +z face is an interface to a neighbouring slab (hg_set_z_interface)
-    int zb;  // z planes per block of the single sweep (0 = default rule; set by the batch autotuner)
+    int zb;  // z planes per block of the single sweep (0 = default rule; pinned by hg_set_block_depth)
     hg::YlmNorm ylm;
     // measurement: kernel launch count and CUDA events around the sub-step kernel
     long long launches;

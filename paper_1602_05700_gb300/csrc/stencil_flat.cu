@@ -4,9 +4,10 @@
 // Measured (Robin, us per sub-step, marching kernels with their own ghost launches -> this one):
 //   compensated float  32^3 14.4 -> 2.4, 64^3 14.4 -> 3.5, 128^3 16.4 -> 8.4, 192^3 46.6 -> 38.0, 256^3 80.7 -> 86
 //   FP64 (1/r field)   32^3 21.2 -> 3.2, 64^3 18.0 -> 5.7, 128^3 39.6 -> 20.8, 192^3 139 -> 68.5, 256^3 228 -> 157
-// (the FP64 figures include the integer forms of lap_int.cuh, and two cells per thread from 600,000 cells).  Blocks of 128 threads: 64 pay for block launches above
-// 96^3, 256 and 512 wait longer for their slowest warp.  2 to 4 planes per thread were no faster anywhere (float 128^3:
-// 9.4, 9.7 and 10.3 us against 9.0): the loads they save hit L2, and they leave fewer threads to cover its latency.
+// (the FP64 figures include the integer forms of lap_int.cuh, and two cells per thread from 600,000 cells).  Blocks of 128
+// threads: 64 pay for block launches above 96^3, 256 and 512 wait longer for their slowest warp.  2 to 4 planes per thread
+// were no faster anywhere (float 128^3: 9.4, 9.7 and 10.3 us against 9.0): the loads they save hit L2, and they leave fewer
+// threads to cover its latency.
 //
 // The adjoint's reverse sub-steps (ADJ) add level n to their running sum from the registers that hold it: a pass of its own
 // took 32 us at 128^3 (float) beside the 9 us of the sub-step; this variant takes 12.

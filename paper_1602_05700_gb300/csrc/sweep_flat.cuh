@@ -1,11 +1,11 @@
 // The flat sweep: one sub-step (arXiv 1602.05700, Sec. 1 Eq. HNeq., Sec. 2: k_g wave sub-steps per hydro step) with a thread
-// of its own for every group of cells (4 of a row for the compensated floats, 1 for FP64), no marching and no shared
+// of its own for every group of cells (4 of a row for the compensated floats, 1 or 2 for FP64), no marching and no shared
 // memory.  All FP64 sub-steps, those of float grids up to 224^3, the adjoint's and the batched launches run it
 // (stencil_flat.cu, batch kernels in stencil.cu).
 //
 // A block that marches in z pays its planes one after the other and keeps few warps resident (the FP64 sweep it replaces:
 // 108 registers, 16 warps per SM).  Here all neighbours of a group are loaded at once, a small grid is one round of
-// loads, one update and one round of stores, and a large FP64 grid has 40 warps per SM to cover the latencies of the FP64
+// loads, one update and one round of stores, and a large FP64 grid has 28 warps of 64 cells per SM to cover the latencies of the FP64
 // and integer pipes that bound it.  The y and z neighbours are re-read through L1 and L2 (46 bytes of L2 traffic per float
 // cell against 30 for the staged sweep, which is why large float grids keep that one).
 //
