@@ -239,7 +239,7 @@ int autotune(hg_batch* b, int budget, int* taken) {
     cudaEventDestroy(e1);
     if (rc) return rc;
     b->zb = 1;
-    b->zb32 = best.zb32;  // without the budget to time anything, the first candidate
+    b->zb32 = best.zb32;  // too few sub-steps to time anything: the first candidate
     b->split = best.split;
     if (complete) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
