@@ -5,23 +5,25 @@
 // a double-double sum costs about 240 FP64 operations per cell at lmax = 4 (9.3 ms at 256^3, against 1.5 ms for the 20
 // sub-steps that follow).  r^l Y_lm is a homogeneous polynomial with integer coefficients up to one factor, so the sums can
 // be taken axis by axis and the harmonics formed once per block:
-//   * a lane owns a row (fixed j, k); 16 consecutive cells at a time it forms the local moments about their centre
-//     from sums and differences of mirrored cells (7 operations per pair at lmax = 4, the factors u^a being integers
-//     <= 15^8), shifts them to the grid's coordinates and adds them to the row's T_a (double-double): 6 per cell;
+//   * a lane owns a row (fixed j, k) and sums rho X^a over it, four cells at a time in plain FP64 and from there on in
+//     double-double (T_a): 9 operations per cell at lmax = 4.  X is the same for all lanes, so its powers come from a table in
+//     shared memory, each rounded once;
 //   * T_a times Z^c goes to the lane's sums over k (10 per row and (a, c)); Y^b, a transposing warp reduction (31 merges
-//     per 32 moments), the sum over warps and the change to Q_lm follow once per block.
-// Coordinates are in half cells about the grid's centre, X = 2 i + 1 - nx, so that every power is an exact integer and the
-// cancellation inside a harmonic (x^2 - y^2 of a round source) is exact.  All sums that cross a group of 16 cells are
-// double-double, and the Cartesian moments stay so through the shift to the origin and the change to Q_lm.
-// Lanes read rows of their own, 16 bytes at a time and a group ahead: the sectors are used whole out of L1, and 32
-// wavefronts per load are 13 us of the 256^3 launch, hidden under the FP64 work.  Float input becomes double by integer
-// instructions (exact), since conversions are slow as well; groups of zeros (vacuum around the source) are skipped.
+//     per 32 moments), the sum over warps and the change to Q_lm follow once per block.  Y^b and Z^c are pairs.
+// Coordinates are half cells counted from the integer one nearest the expansion origin, so a term is no larger than the moment
+// it belongs to (counted from the grid's centre, a compact source at an origin off the centre lost (distance / radius)^l of its
+// accuracy: 7e6 units of 2^-53 sum |rho| |x|^l at l = 8), the powers are integers (exact up to 2^53) and the cancellation inside
+// a harmonic (x^2 - y^2 of a round source) holds.  The Cartesian moments stay pairs through the shift by the remaining half
+// cell or less to the origin and the change to Q_lm.
+// Lanes read rows of their own, 16 cells at a time and a group ahead: the sectors are used whole out of L1.  Float input
+// becomes double by integer instructions (exact), since conversions are slow as well; groups of zeros (vacuum around the
+// source) are skipped.
 //
-// Measured (random density, us, harmonics per cell -> this): lmax 4: 32^3 155 -> 64, 128^3 1190 -> 102, 256^3 9316 ->
-// 361 (FP64 work alone: 220; the reduction and the change of basis are a fixed 60 of latency); lmax 8 at 256^3 30,000 ->
-// 848; lmax 0 at 256^3 350 -> 115.  Error against quad precision (largest over spheres, blobs, constants and noise,
-// centred and shifted origins, lmax 4 and 8, relative to the largest moment / to the largest of the same degree):
-// 3.2e-16 / 5.3e-15 -> 2.4e-16 / 1.6e-15.
+// Measured (random density, a call of hg_moments_noalloc with both its launches, us, harmonics per cell -> this): lmax 4:
+// 32^3 347 -> 74, 128^3 1475 -> 121, 256^3 9490 -> 450, 512^3 73,500 -> 2790; lmax 8: 256^3 30,030 -> 921; lmax 0: 256^3 374 ->
+// 115.  (Sums of 16 cells in plain FP64 about the grid's centre: 407 at 256^3 and lmax 4.)  Error in units of 2^-53 sum |rho| |x|^l
+// over spheres, Gaussians, constants and noise, centred or up to 0.8 of the way to a face, lmax 4 and 8 (the kernel's order
+// evaluated on the host against quad precision; harmonics per cell with an exact sum -> this): largest 0.74 -> 0.44.
 #pragma once
 
 #include "cell.cuh"
@@ -72,10 +74,13 @@ static __device__ const HarmonicTable kHarmonics = make_harmonics();
 // rounding error that the lossless scheme then carries, through the Dirichlet data, into phi; so every partial sum
 // is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding errors), whose
 // error is of order n eps^2 of the sum of |terms|.
+// TwoSum as FastTwoSum on the operands ordered by the high words of their magnitudes (so the first one's exponent is not the
+// smaller): three FP64 operations and integer selects, where TwoSum takes six on the pipe that bounds the kernel.
 __device__ __forceinline__ void dd_add(double& s, double& e, double x) {
-    const double t = __dadd_rn(s, x);
-    const double v = __dsub_rn(t, s);
-    e = __dadd_rn(e, __dadd_rn(__dsub_rn(s, __dsub_rn(t, v)), __dsub_rn(x, v)));
+    const bool swap = (__double2hiint(s) & 0x7fffffff) < (__double2hiint(x) & 0x7fffffff);
+    const double a = swap ? x : s, b = swap ? s : x;
+    const double t = __dadd_rn(a, b);
+    e = __dadd_rn(e, __dsub_rn(b, __dsub_rn(t, a)));
     s = t;
 }
 // (s, e) += (s2, e2), renormalised so that s is the rounded value of the pair
@@ -104,55 +109,58 @@ __device__ __forceinline__ void dd_warp(double& s, double& e) {
 __device__ __forceinline__ bool nonzero(float x) { return (__float_as_uint(x) << 1) != 0u; }
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 
-constexpr int kMomGroup = 16;  // cells of a row taken together
+constexpr int kMomGroup = 16;  // cells of a row loaded together
+constexpr int kMomSum = 4;     // cells summed in plain FP64
+constexpr int kMomStretch = 2048;  // most cells of a row in the table of powers (8 x 16 KB at lmax = 8)
 
-// the 16 cells of a row from cell `start` on; those before `lo` or beyond `hi` are 0.  vec: the row starts on a 16-byte
-// boundary and has a whole number of 16-byte words, so that a group inside it can be read in such words
-__device__ __forceinline__ void mom_load(const float* __restrict__ row, int start, int lo, int hi, bool vec,
-                                         float (&v)[kMomGroup]) {
-    if (vec && start >= 0 && start + kMomGroup <= hi) {
+// the 16 cells of a row from cell `start` on; those beyond `hi` are 0.  vec: the row starts on a 16-byte boundary and has a
+// whole number of 16-byte words, so that a group inside it can be read in such words
+__device__ __forceinline__ void mom_load(const float* __restrict__ row, int start, int hi, bool vec, float (&v)[kMomGroup]) {
+    if (vec && start + kMomGroup <= hi) {
 #pragma unroll
         for (int g = 0; g < kMomGroup; g += 4) {
             const float4 x = __ldg(reinterpret_cast<const float4*>(row + start + g));
             v[g] = x.x, v[g + 1] = x.y, v[g + 2] = x.z, v[g + 3] = x.w;
         }
-        if (start < lo)
-#pragma unroll
-            for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo ? v[e] : 0.f;
     } else {
 #pragma unroll
-        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo && start + e < hi ? __ldg(row + start + e) : 0.f;
+        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e < hi ? __ldg(row + start + e) : 0.f;
     }
 }
-__device__ __forceinline__ void mom_load(const double* __restrict__ row, int start, int lo, int hi, bool vec,
-                                         double (&v)[kMomGroup]) {
-    if (vec && start >= 0 && start + kMomGroup <= hi) {
+__device__ __forceinline__ void mom_load(const double* __restrict__ row, int start, int hi, bool vec, double (&v)[kMomGroup]) {
+    if (vec && start + kMomGroup <= hi) {
 #pragma unroll
         for (int g = 0; g < kMomGroup; g += 2) {
             const double2 x = __ldg(reinterpret_cast<const double2*>(row + start + g));
             v[g] = x.x, v[g + 1] = x.y;
         }
-        if (start < lo)
-#pragma unroll
-            for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo ? v[e] : 0.0;
     } else {
 #pragma unroll
-        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e >= lo && start + e < hi ? __ldg(row + start + e) : 0.0;
+        for (int e = 0; e < kMomGroup; ++e) v[e] = start + e < hi ? __ldg(row + start + e) : 0.0;
     }
 }
 
 struct MomArgs {
     int nx, ny, nz;
     double h3[2];              // cell volume, as a pair
-    double off[3][2];          // offset of the grid's centre from the origin in half cells, as a pair, per axis
+    double org[3];             // the integer half cell nearest the origin, counted from the grid's corner, per axis
+    double off[3][2];          // offset of that half cell from the origin in half cells (at most 1/2), as a pair
     double hl[kMaxL + 1][2];   // (h / 4)^l as a pair: half cells and the table's 2^-l
     int centred;               // off is zero
 };
 
+// (p, pe) <- (p, pe) * X for an integer X: exact while the power is below 2^106
+__device__ __forceinline__ void dd_power(double& p, double& pe, double X) {
+    const double q = __dmul_rn(p, X);
+    pe = __fma_rn(pe, X, __fma_rn(p, X, -q));
+    p = q;
+}
+
 // per-block partial moments: partial[2 (block nq + q) + {0, 1}]
 template <typename T, int LMAX>
 __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restrict__ rho, bool vec, MomArgs P,
-                                                               YlmNorm N, double* __restrict__ partial) {
+                                                               YlmNorm N, double* __restrict__ partial, int ch) {
+    extern __shared__ __align__(16) double pw[];  // [a][ch], a < LMAX: X^(a+1) of the cells of a stretch of the rows
     constexpr int NQ = (LMAX + 1) * (LMAX + 1), NM = mono_off(LMAX + 1), NB = (NM + 31) / 32;
     __shared__ double wm[kMomWarps][NB * 32][2], tot[NM][2], moved[NM][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -160,118 +168,124 @@ __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restri
     // tasks: (32 rows, 1 plane), plane fastest; a warp takes a contiguous range, so that its rows stay the same
     const long long tasks = (long long)((P.ny + 31) / 32) * P.nz, W = (long long)kMomBlocks * kMomWarps;
     const long long w = (long long)blockIdx.x * kMomWarps + warp;
-    long long t = w * tasks / W;
-    const long long t1 = (w + 1) * tasks / W;
-    while (t < t1) {
-        const int jg = (int)(t / P.nz), k0 = (int)(t % P.nz);
-        const int k1 = (int)(t1 - t < P.nz - k0 ? k0 + (t1 - t) : P.nz);
-        t += k1 - k0;
-        const int j = jg * 32 + lane;
-        const bool mine = j < P.ny;
-        double As[LMAX + 1][LMAX + 1], Ae[LMAX + 1][LMAX + 1];  // [a][c], a + c <= LMAX
+    for (int x0 = 0; x0 < P.nx; x0 += ch) {
+        const int x1 = P.nx < x0 + ch ? P.nx : x0 + ch;
+        if constexpr (LMAX > 0) {
+            __syncthreads();  // the stretch before is done with
+            for (int i = threadIdx.x; i < ((x1 - x0 + kMomGroup - 1) & -kMomGroup); i += 32 * kMomWarps) {
+                const double X = (double)(2ll * (x0 + i) + 1) - P.org[0];
+                double p = X, pe = 0.0;
 #pragma unroll
-        for (int a = 0; a <= LMAX; ++a)
-#pragma unroll
-            for (int c = 0; c <= LMAX; ++c) As[a][c] = Ae[a][c] = 0.0;
-        for (int k = k0; k < k1; ++k) {
-            const T* row = rho + ((long long)k * P.ny + (mine ? j : 0)) * P.nx;
-            double Ts[LMAX + 1], Te[LMAX + 1];
-#pragma unroll
-            for (int a = 0; a <= LMAX; ++a) Ts[a] = Te[a] = 0.0;
-            // groups of 16 cells; the last one ends with the row (its cells that belong to the one before are masked), and
-            // a row shorter than a group sits in the group's middle: a group never reaches beyond the row, so its local
-            // powers are no larger than the row's own
-            const int ng = (P.nx + kMomGroup - 1) / kMomGroup, hi = mine ? P.nx : 0;
-            auto start_of = [&](int g) {
-                return g < ng - 1 ? g * kMomGroup : P.nx >= kMomGroup ? P.nx - kMomGroup : -((kMomGroup - P.nx) / 2);
-            };
-            T nv[kMomGroup];  // the next group's cells: in flight while this one is worked on
-            mom_load(row, start_of(0), 0, hi, vec, nv);
-            for (int g = 0; g < ng; ++g) {
-                const int i = start_of(g);
-                T v[kMomGroup];
-#pragma unroll
-                for (int e = 0; e < kMomGroup; ++e) v[e] = nv[e];
-                if (g + 1 < ng) mom_load(row, start_of(g + 1), (g + 1) * kMomGroup, hi, vec, nv);
-                bool any = false;
-#pragma unroll
-                for (int e = 0; e < kMomGroup; ++e) any = any || nonzero(v[e]);
-                if (!__any_sync(0xffffffffu, any)) continue;
-                double loc[LMAX + 1];
-#pragma unroll
-                for (int a = 0; a <= LMAX; ++a) loc[a] = 0.0;
-#pragma unroll
-                for (int p = 0; p < kMomGroup / 2; ++p) {  // the cells at -u and +u half cells from the group's centre
-                    const double u = kMomGroup - 1 - 2 * p;
-                    const double lo = widen(v[p]), hi = widen(v[kMomGroup - 1 - p]);
-                    const double s = __dadd_rn(lo, hi);
-                    const double d = LMAX ? __dsub_rn(hi, lo) : 0.0;
-                    double f = 1.0;
-#pragma unroll
-                    for (int a = 0; a <= LMAX; ++a) {
-                        loc[a] = __fma_rn((a & 1) ? d : s, f, loc[a]);
-                        f *= u;
-                    }
-                }
-                // about the group's centre -> the grid's coordinates: loc_a <- sum_b C(a, b) X^(a-b) loc_b
-                const double X = (double)(2 * i + kMomGroup - P.nx);
-#pragma unroll
-                for (int b = 1; b <= LMAX; ++b)
-#pragma unroll
-                    for (int a = LMAX; a >= b; --a) loc[a] = __fma_rn(X, loc[a - 1], loc[a]);
-#pragma unroll
-                for (int a = 0; a <= LMAX; ++a) dd_add(Ts[a], Te[a], loc[a]);
-            }
-            const double Z = (double)(2 * k + 1 - P.nz);
-            double zc = 1.0;
-#pragma unroll
-            for (int c = 0; c <= LMAX; ++c) {
-#pragma unroll
-                for (int a = 0; a + c <= LMAX; ++a) dd_fma(As[a][c], Ae[a][c], Ts[a], Te[a], zc);
-                zc *= Z;
-            }
-        }
-        // times Y^b, summed over the warp's rows: each step halves the lanes a moment is spread over and the moments a
-        // lane holds, so lane n ends with moment n of the batch
-        if constexpr (NM == 1) {
-            dd_warp(As[0][0], Ae[0][0]);
-            if (lane == 0) dd_merge(wm[warp][0][0], wm[warp][0][1], As[0][0], Ae[0][0]);
-            continue;
-        }
-        const double Y = (double)(2 * j + 1 - P.ny);
-        double yb[LMAX + 1];
-        yb[0] = 1.0;
-#pragma unroll
-        for (int b = 1; b <= LMAX; ++b) yb[b] = yb[b - 1] * Y;
-#pragma unroll
-        for (int B = 0; B < NB; ++B) {
-            double vs[32], ve[32];
-#pragma unroll
-            for (int n = 0; n < 32; ++n) vs[n] = ve[n] = 0.0;
-#pragma unroll
-            for (int l = 0; l <= LMAX; ++l)
-#pragma unroll
-                for (int c = 0; c <= l; ++c)
-#pragma unroll
-                    for (int b = 0; b + c <= l; ++b) {
-                        const int n = mono_off(l) + mono_at(l, b, c) - 32 * B;
-                        if (n >= 0 && n < 32) dd_fma(vs[n], ve[n], As[l - b - c][c], Ae[l - b - c][c], yb[b]);
-                    }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const bool up = lane & o;
-#pragma unroll
-                for (int n = 0; n < o; ++n) {
-                    const double s2 = __shfl_xor_sync(0xffffffffu, up ? vs[n] : vs[n + o], o);
-                    const double e2 = __shfl_xor_sync(0xffffffffu, up ? ve[n] : ve[n + o], o);
-                    if (up) {
-                        vs[n] = vs[n + o];
-                        ve[n] = ve[n + o];
-                    }
-                    dd_merge(vs[n], ve[n], s2, e2);
+                for (int a = 0; a < LMAX; ++a) {
+                    pw[a * ch + i] = __dadd_rn(p, pe);
+                    dd_power(p, pe, X);
                 }
             }
-            dd_merge(wm[warp][32 * B + lane][0], wm[warp][32 * B + lane][1], vs[0], ve[0]);
+            __syncthreads();
+        }
+        long long t = w * tasks / W;
+        const long long t1 = (w + 1) * tasks / W;
+        while (t < t1) {
+            const int jg = (int)(t / P.nz), k0 = (int)(t % P.nz);
+            const int k1 = (int)(t1 - t < P.nz - k0 ? k0 + (t1 - t) : P.nz);
+            t += k1 - k0;
+            const int j = jg * 32 + lane;
+            const bool mine = j < P.ny;
+            double As[LMAX + 1][LMAX + 1], Ae[LMAX + 1][LMAX + 1];  // [a][c], a + c <= LMAX
+#pragma unroll
+            for (int a = 0; a <= LMAX; ++a)
+#pragma unroll
+                for (int c = 0; c <= LMAX; ++c) As[a][c] = Ae[a][c] = 0.0;
+            for (int k = k0; k < k1; ++k) {
+                const T* row = rho + ((long long)k * P.ny + (mine ? j : 0)) * P.nx;
+                const int hi = mine ? x1 : 0;
+                double Ts[LMAX + 1], Te[LMAX + 1];
+#pragma unroll
+                for (int a = 0; a <= LMAX; ++a) Ts[a] = Te[a] = 0.0;
+                T nv[kMomGroup];  // the next group's cells: in flight while this one is worked on
+                mom_load(row, x0, hi, vec, nv);
+                for (int i = x0; i < x1; i += kMomGroup) {
+                    T v[kMomGroup];
+#pragma unroll
+                    for (int e = 0; e < kMomGroup; ++e) v[e] = nv[e];
+                    if (i + kMomGroup < x1) mom_load(row, i + kMomGroup, hi, vec, nv);
+                    bool any = false;
+#pragma unroll
+                    for (int e = 0; e < kMomGroup; ++e) any = any || nonzero(v[e]);
+                    if (!__any_sync(0xffffffffu, any)) continue;
+#pragma unroll
+                    for (int g = 0; g < kMomGroup; g += kMomSum) {
+                        double c[kMomSum];
+#pragma unroll
+                        for (int e = 0; e < kMomSum; ++e) c[e] = widen(v[g + e]);
+#pragma unroll
+                        for (int a = 0; a <= LMAX; ++a) {
+                            double s;
+                            if (a == 0) {
+                                s = __dadd_rn(__dadd_rn(c[0], c[1]), __dadd_rn(c[2], c[3]));
+                            } else {
+                                const double2* p = reinterpret_cast<const double2*>(pw + (a - 1) * ch + (i - x0 + g));
+                                const double2 pa = p[0], pb = p[1];
+                                s = __fma_rn(c[3], pb.y, __fma_rn(c[2], pb.x, __fma_rn(c[1], pa.y, __dmul_rn(c[0], pa.x))));
+                            }
+                            dd_add(Ts[a], Te[a], s);
+                        }
+                    }
+                }
+                const double Z = (double)(2ll * k + 1) - P.org[2];
+                double zc = 1.0, ze = 0.0;
+#pragma unroll
+                for (int c = 0; c <= LMAX; ++c) {
+#pragma unroll
+                    for (int a = 0; a + c <= LMAX; ++a) dd_fma(As[a][c], Ae[a][c], Ts[a], Te[a], zc, ze);
+                    dd_power(zc, ze, Z);
+                }
+            }
+            // times Y^b, summed over the warp's rows: each step halves the lanes a moment is spread over and the moments a
+            // lane holds, so lane n ends with moment n of the batch
+            if constexpr (NM == 1) {
+                dd_warp(As[0][0], Ae[0][0]);
+                if (lane == 0) dd_merge(wm[warp][0][0], wm[warp][0][1], As[0][0], Ae[0][0]);
+                continue;
+            }
+            const double Y = (double)(2ll * j + 1) - P.org[1];
+            double yb[LMAX + 1], ye[LMAX + 1];
+            yb[0] = 1.0, ye[0] = 0.0;
+#pragma unroll
+            for (int b = 1; b <= LMAX; ++b) {
+                yb[b] = yb[b - 1], ye[b] = ye[b - 1];
+                dd_power(yb[b], ye[b], Y);
+            }
+#pragma unroll
+            for (int B = 0; B < NB; ++B) {
+                double vs[32], ve[32];
+#pragma unroll
+                for (int n = 0; n < 32; ++n) vs[n] = ve[n] = 0.0;
+#pragma unroll
+                for (int l = 0; l <= LMAX; ++l)
+#pragma unroll
+                    for (int c = 0; c <= l; ++c)
+#pragma unroll
+                        for (int b = 0; b + c <= l; ++b) {
+                            const int n = mono_off(l) + mono_at(l, b, c) - 32 * B;
+                            if (n >= 0 && n < 32) dd_fma(vs[n], ve[n], As[l - b - c][c], Ae[l - b - c][c], yb[b], ye[b]);
+                        }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const bool up = lane & o;
+#pragma unroll
+                    for (int n = 0; n < o; ++n) {
+                        const double s2 = __shfl_xor_sync(0xffffffffu, up ? vs[n] : vs[n + o], o);
+                        const double e2 = __shfl_xor_sync(0xffffffffu, up ? ve[n] : ve[n + o], o);
+                        if (up) {
+                            vs[n] = vs[n + o];
+                            ve[n] = ve[n + o];
+                        }
+                        dd_merge(vs[n], ve[n], s2, e2);
+                    }
+                }
+                dd_merge(wm[warp][32 * B + lane][0], wm[warp][32 * B + lane][1], vs[0], ve[0]);
+            }
         }
     }
     __syncthreads();
@@ -282,7 +296,7 @@ __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restri
         tot[m][1] = e;
     }
     __syncthreads();
-    if (!P.centred) {  // about the grid's centre -> about the origin, one axis after the other (binomials)
+    if (!P.centred) {  // about the half cell -> about the origin, one axis after the other (binomials)
         for (int axis = 0; axis < 3; ++axis) {
             for (int m = threadIdx.x; m < NM; m += 32 * kMomWarps) {
                 int l = 0, b = m, c = 0;
@@ -349,13 +363,11 @@ cudaError_t launch_moments(const void* rho, int dtype, int nx, int ny, int nz, d
     P.h3[0] = h2 * h;
     P.h3[1] = fma(h2, h, -P.h3[0]) + h2e * h;
     P.centred = 1;
-    const int ext[3] = {nx, ny, nz};
-    for (int a = 0; a < 3; ++a) {  // 2 (o + n h / 2) / h, product, sum and quotient each with its rounding error
-        const double hn = 0.5 * ext[a], p = hn * h, pe = fma(hn, h, -p);
-        const double t = p + o[a], v = t - p, te = ((p - (t - v)) + (o[a] - v)) + pe;
-        const double q = 2.0 * t / h;
-        P.off[a][0] = q;
-        P.off[a][1] = (fma(-q, h, 2.0 * t) + 2.0 * te) / h;
+    for (int a = 0; a < 3; ++a) {  // 2 o / h: the quotient and its rounding error, less the integer next to it (exact)
+        const double q = 2.0 * o[a] / h;
+        P.org[a] = -nearbyint(q);
+        P.off[a][0] = q + P.org[a];
+        P.off[a][1] = fma(-q, h, 2.0 * o[a]) / h;
         if (P.off[a][0] != 0.0 || P.off[a][1] != 0.0) P.centred = 0;
     }
     P.hl[0][0] = 1.0, P.hl[0][1] = 0.0;
@@ -367,11 +379,21 @@ cudaError_t launch_moments(const void* rho, int dtype, int nx, int ny, int nz, d
     const int per16 = dtype == HG_DT_F64 ? 2 : 4;
     const bool vec = nx % per16 == 0 && (uintptr_t)rho % 16 == 0;
     const int th = 32 * kMomWarps;
+    const int ch = nx < kMomStretch ? (nx + kMomGroup - 1) & -kMomGroup : kMomStretch;
+    const int smem = LMAX * ch * (int)sizeof(double);
+    constexpr int NM = mono_off(LMAX + 1), held = 16 * (kMomWarps * ((NM + 31) / 32) * 32 + 2 * NM);  // static part
+    cudaError_t e = cudaSuccess;
+    auto launch = [&](auto* kernel, const auto* r) {
+        if (held + smem > 48 * 1024)  // above 48 KB a kernel has to ask (each time: a device reset forgets it)
+            e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return;
+        kernel<<<kMomBlocks, th, smem, st>>>(r, vec, P, N, scratch, ch);
+        e = cudaGetLastError();
+    };
     if (dtype == HG_DT_F64)
-        k_moments<double, LMAX><<<kMomBlocks, th, 0, st>>>((const double*)rho, vec, P, N, scratch);
+        launch(k_moments<double, LMAX>, (const double*)rho);
     else
-        k_moments<float, LMAX><<<kMomBlocks, th, 0, st>>>((const float*)rho, vec, P, N, scratch);
-    cudaError_t e = cudaGetLastError();
+        launch(k_moments<float, LMAX>, (const float*)rho);
     if (e != cudaSuccess) return e;
     k_finish_moments<<<NQ, 32, 0, st>>>(scratch, NQ, Q);
     return cudaGetLastError();
