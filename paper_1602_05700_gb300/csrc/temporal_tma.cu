@@ -83,17 +83,22 @@ __device__ __forceinline__ void robin4(const Bnd& B, int f, long long t0, const 
     }
 }
 
-// One block.  WHOLE: every tile is 128 cells wide -- nx >= 128 is a multiple of 8, and where it is not one of 128 the last tile
-// starts at nx - 128 and shares columns with its neighbour (both compute and store the same values; a bulk copy of the
-// 16-bit codes has to start on a multiple of 8 cells) -- so that the x halo columns are always the helper's.  Otherwise the
+// How the tiles cover a row.  kWhole and kShared: every tile is 128 cells wide -- nx >= 128 is a multiple of 128, or (kShared) of
+// 8, and then the last tile starts at nx - 128 and computes again, but does not store, the columns that belong to its
+// neighbour (a bulk copy of the 16-bit codes has to start on a multiple of 8 cells; the two blocks round some of those columns
+// by different forms of the update, and a cell's hi, code and increment have to come from one block; in kWhole tiles the test of
+// a column's owner would cost 512^3 1.7%) -- so that the x halo columns are always the helper's.  Otherwise the
 // last tile may be ragged, with the +x ghost inside it, in one lane of each row warp; all tiles then run that more general
 // code: with a copy of each kind in one kernel the blocks that share an SM fetched more instructions than its cache holds
 // (52% of all stall cycles on a grid with ragged tiles).
-template <bool WHOLE, bool EXACT>
+enum Tiles { kGeneral, kWhole, kShared };
+
+template <Tiles TILES, bool EXACT>
 __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUtensorMap* m_lo, const CUtensorMap* m_d,
                                              const CUtensorMap* m_s, const SweepArgs& A, float* __restrict__ d_out,
                                              int* err, unsigned char* smem, unsigned long long* bar_full,
                                              volatile int* abort_flag) {
+    constexpr bool WHOLE = TILES != kGeneral;
     const Layout& L = A.L;
     const Bnd& B = A.B;
     const bool robin = B.faces != 0;
@@ -229,6 +234,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     const int xa = x0 + 4 * lane;  // first cell of this lane's group
     const int col = 4 + 4 * lane;  // its stage / ring column
     const int nlive = WHOLE ? 4 : max(0, min(4, L.nx - xa));  // interior cells of the group
+    const bool own = TILES != kShared || xa >= (int)blockIdx.x * kFX;  // not a column that the tile before stores
     // the element of the group that is the +x ghost, or -1 (in a ragged tile one lane of each row warp has it)
     const int ge = !WHOLE && L.nx >= xa && L.nx < xa + 4 ? L.nx - xa : -1;
     // the ghost's value of the next level from the group's values (h, l) and the cell before the group (xl, ll): unchanged
@@ -339,7 +345,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
         float4 ho, lo;
         robin4(B, R.y < 0 ? 2 : 3, (long long)q * L.nx + xa, hg, lg, gin, lgin, ho, lo, nlive);
         const long long qo = L.at(xa, R.y, q);
-        if (!idx_ok(qo, nlive, L.elems, B.err)) return;
+        if (!own || !idx_ok(qo, nlive, L.elems, B.err)) return;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             if (e < nlive) {
@@ -432,7 +438,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
                 else
                     f32k_update4(c1, lc1, gl, gll, gr, grl, ys, yn, m1, h1, lys, lyn, lm1, l1, d1c, sc, nu2, ho, lo, dout);
                 const long long qo = L.at(xa, y, q);
-                if (!idx_ok(qo, 4, L.elems, B.err)) {
+                if (!own || !idx_ok(qo, 4, L.elems, B.err)) {
                 } else if (WHOLE || nlive == 4) {
                     *reinterpret_cast<float4*>(hi_n + qo) = ho;
                     *reinterpret_cast<uint2*>(lo_n + qo) = lo_encode4(ho, lo);
@@ -465,7 +471,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
                 const long long qo = L.at(xa, y, lo_face ? -1 : L.nz);
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if (e < nlive && idx_ok(qo + e, 1, L.elems, B.err)) {
+                    if (e < nlive && own && idx_ok(qo + e, 1, L.elems, B.err)) {
                         hi_n[qo + e] = el(ho, e);
                         lo_n[qo + e] = lo_encode(el(ho, e), el(lo, e));
                     }
@@ -484,7 +490,7 @@ __device__ __forceinline__ void fused2_block(const CUtensorMap* m_hi, const CUte
     }
 }
 
-template <bool WHOLE, bool EXACT>
+template <Tiles TILES, bool EXACT>
 __global__ void __maxnreg__(96)  // 2 blocks of 320 threads per SM (5 warps of 96 registers per SM quarter)
     k_temporal2_tma(const __grid_constant__ CUtensorMap m_hi, const __grid_constant__ CUtensorMap m_lo,
                     const __grid_constant__ CUtensorMap m_d, const __grid_constant__ CUtensorMap m_s,
@@ -501,7 +507,7 @@ __global__ void __maxnreg__(96)  // 2 blocks of 320 threads per SM (5 warps of 9
     __syncthreads();
     pdl_trigger();
     pdl_wait();
-    fused2_block<WHOLE, EXACT>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
+    fused2_block<TILES, EXACT>(&m_hi, &m_lo, &m_d, &m_s, A, d_out, err, smem, bar_full, &abort_flag);
 }
 
 constexpr int kZ2 = F2::planes;  // level-(n+2) planes per block
@@ -539,13 +545,15 @@ int launch_temporal2_tma(hg_grid* g) {
     // against 471 before the copies went first), except in exact mode on grids of more than one wave of blocks, where the general code comes out
     // faster (512^3: 483 against 521 us; the register allocation of the scalar update differs), not on smaller ones
     // (128^3: 32 against 37)
-    const bool whole = g->nx >= kFX && g->nx % 8 == 0;
-    const int v = g->texact ? (whole && (long long)grid.x * grid.y * grid.z <= 304 ? 0 : 1) : whole ? 2 : 3;
-    static unsigned long long attr_done[4] = {0, 0, 0, 0};
-    const auto kernel = v == 0   ? k_temporal2_tma<true, true>
-                        : v == 1 ? k_temporal2_tma<false, true>
-                        : v == 2 ? k_temporal2_tma<true, false>
-                                 : k_temporal2_tma<false, false>;
+    const bool whole = g->nx >= kFX && g->nx % 8 == 0 && !(g->texact && (long long)grid.x * grid.y * grid.z > 304);
+    const int v = (!whole ? 0 : g->nx % kFX == 0 ? 1 : 2) + (g->texact ? 3 : 0);
+    static unsigned long long attr_done[6] = {0, 0, 0, 0, 0, 0};
+    const auto kernel = v == 0   ? k_temporal2_tma<kGeneral, false>
+                        : v == 1 ? k_temporal2_tma<kWhole, false>
+                        : v == 2 ? k_temporal2_tma<kShared, false>
+                        : v == 3 ? k_temporal2_tma<kGeneral, true>
+                        : v == 4 ? k_temporal2_tma<kWhole, true>
+                                 : k_temporal2_tma<kShared, true>;
     if ((rc = smem_attr_once((const void*)kernel, F2::smem, &attr_done[v]))) return rc;
     if ((rc = prof_begin(g))) return rc;
     if ((rc = launch_pdl(kernel, grid, dim3(kFThreads), F2::smem, g->stream, g->tm2[0 + c], g->tm2[2 + c],
