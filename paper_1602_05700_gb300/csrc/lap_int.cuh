@@ -129,6 +129,23 @@ __host__ __device__ __forceinline__ Lap6 lap6_units(double c, double x0, double 
     return r;
 }
 
+// The values at p and p + 1 (p on 16 bytes), or the one at p twice where `two` is false: behind the last cell of an odd row lies
+// the +x ghost, which another thread of the launch may be writing, so it is not read there.
+__host__ __device__ __forceinline__ void load_pair(const double* p, bool two, double (&v)[2]) {
+    if (two) {
+#ifdef __CUDA_ARCH__
+        const double2 x = *reinterpret_cast<const double2*>(p);
+        v[0] = x.x;
+        v[1] = x.y;
+#else
+        v[0] = p[0];
+        v[1] = p[1];
+#endif
+    } else {
+        v[0] = v[1] = p[0];
+    }
+}
+
 // Two cells next to each other along x in common units (the smallest ulp of their twelve values): the conversions of c0, c1
 // and their difference serve both.  v[q]: the neighbours of cell q in the order of the sum (v[0][1] is c1, v[1][0] is c0).
 struct Lap6Pair {

@@ -3,7 +3,7 @@
 //
 // Measured (Robin, us per sub-step, marching kernels with their own ghost launches -> this one):
 //   compensated float  32^3 14.4 -> 2.4, 64^3 14.4 -> 3.5, 128^3 16.4 -> 8.4, 192^3 46.6 -> 38.0, 256^3 80.7 -> 86
-//   FP64 (1/r field)   32^3 21.2 -> 3.2, 64^3 18.0 -> 5.7, 128^3 39.6 -> 20.8, 192^3 139 -> 68.5, 256^3 228 -> 157
+//   FP64 (1/r field)   32^3 21.2 -> 3.2, 64^3 18.0 -> 5.7, 128^3 39.6 -> 20.6, 192^3 139 -> 67.4, 256^3 228 -> 155
 // (the FP64 figures include the integer forms of lap_int.cuh, and two cells per thread from 600,000 cells).  Blocks of 128
 // threads: 64 pay for block launches above 96^3, 256 and 512 wait longer for their slowest warp.  2 to 4 planes per thread
 // were no faster anywhere (float 128^3: 9.4, 9.7 and 10.3 us against 9.0): the loads they save hit L2, and they leave fewer
@@ -23,8 +23,8 @@ constexpr int kFlatThreads = 128;
 
 // FP64: two cells per thread from here on.  They share the conversions of the integer forms (198 instructions per cell
 // instead of 248) and move 16 bytes per access; smaller grids want the threads.  Measured, us per sub-step, one -> two cells:
-// 32^3 2.59 -> 4.1, 64^3 4.82 -> 4.82, 96^3 10.9 -> 10.5, 128^3 22.6 -> 20.8, 192^3 75.4 -> 68.5, 256^3 176 -> 157,
-// 301x259x223 184 -> 163.  (Marching 2 to 16 planes per thread, with or without square tiles, 144-150 us in a field where this
+// 32^3 2.59 -> 4.1, 64^3 4.82 -> 4.82, 96^3 10.9 -> 10.5, 128^3 22.6 -> 20.6, 192^3 75.4 -> 67.4, 256^3 176 -> 155,
+// 301x259x223 184 -> 165.  (Marching 2 to 16 planes per thread, with or without square tiles, 144-150 us in a field where this
 // takes 148: the loads it saves do not bound it.)  The adjoint's reverse sub-steps keep one cell per thread: their injection is
 // sparse, and a warp of 64 cells is oftener left to FP64 (128^3 adjoint 10.6 against 11.2 ms).
 constexpr long long kPairCells = 600000;
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(kFlatThreads, 10) k_step_f64(const SweepArgs A
 }
 
 // 7 resident blocks of 72 registers; 6 and 8 (spills) are both 3-8% slower
-template <bool WIDE>
+template <bool ODD, bool WIDE>
 __global__ void __launch_bounds__(kFlatThreads, 7) k_step_f64x2(const SweepArgs A, const FlatGrid G) {
     pdl_trigger();
     if (blockIdx.x < G.ghost_tiles) {
@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kFlatThreads, 7) k_step_f64x2(const SweepArgs 
     int i, j, k;
     const bool mine = flat_cell<WIDE>(A.L, G, blockIdx.x, 2, i, j, k);
     pdl_wait();
-    if (mine) flat_f64x2(A, i, j, k);
+    if (mine) flat_f64x2<ODD>(A, i, j, k);
 }
 
 }  // namespace
@@ -97,7 +97,8 @@ int launch_step_flat(hg_grid* g, void* acc_a, void* acc_b) {
             return launch_pdl(k_step_f32k_flat<adj.value, wide.value>, dim3(G.tiles), dim3(kFlatThreads), 0, g->stream, A, G,
                               (float*)acc_a, (float*)acc_b);
         if (pairs)
-            return launch_pdl(k_step_f64x2<wide.value>, dim3(G.tiles), dim3(kFlatThreads), 0, g->stream, A, G);
+            return launch_pdl(g->nx % 2 ? k_step_f64x2<true, wide.value> : k_step_f64x2<false, wide.value>, dim3(G.tiles),
+                              dim3(kFlatThreads), 0, g->stream, A, G);
         return launch_pdl(k_step_f64<adj.value, wide.value>, dim3(G.tiles), dim3(kFlatThreads), 0, g->stream, A, G,
                           (double*)acc_a);
     };
