@@ -5,7 +5,7 @@
 // a double-double sum costs about 240 FP64 operations per cell at lmax = 4 (9.3 ms at 256^3, against 1.5 ms for the 20
 // sub-steps that follow).  r^l Y_lm is a homogeneous polynomial with integer coefficients up to one factor, so the sums can
 // be taken axis by axis and the harmonics formed once per block:
-//   * a lane owns a row (fixed j, k) and sums rho X^a over it, four cells at a time in plain FP64 and from there on in
+//   * a lane owns a row (fixed j, k), or a part of one, and sums rho X^a over it, four cells at a time in plain FP64 and from there on in
 //     double-double (T_a): 9 operations per cell at lmax = 4.  X is the same for all lanes, so its powers come from a table in
 //     shared memory, each rounded once;
 //   * T_a times Z^c goes to the lane's sums over k (10 per row and (a, c)); Y^b, a transposing warp reduction (31 merges
@@ -20,8 +20,8 @@
 // source) are skipped.
 //
 // Measured (random density, a call of hg_moments_noalloc with both its launches, us, harmonics per cell -> this): lmax 4:
-// 32^3 347 -> 74, 128^3 1475 -> 121, 256^3 9490 -> 450, 512^3 73,500 -> 2790; lmax 8: 256^3 30,030 -> 921; lmax 0: 256^3 374 ->
-// 115.  (Sums of 16 cells in plain FP64 about the grid's centre: 407 at 256^3 and lmax 4.)  Error in units of 2^-53 sum |rho| |x|^l
+// 32^3 347 -> 74, 128^3 1475 -> 117, 256^3 9490 -> 449, 512^3 73,500 -> 2790; lmax 8: 256^3 30,030 -> 925; lmax 0: 256^3 374 ->
+// 116.  (Sums of 16 cells in plain FP64 about the grid's centre: 407 at 256^3 and lmax 4.)  Error in units of 2^-53 sum |rho| |x|^l
 // over spheres, Gaussians, constants and noise, centred or up to 0.8 of the way to a face, lmax 4 and 8 (the kernel's order
 // evaluated on the host against quad precision; harmonics per cell with an exact sum -> this): largest 0.74 -> 0.44.
 #pragma once
@@ -142,6 +142,7 @@ __device__ __forceinline__ void mom_load(const double* __restrict__ row, int sta
 
 struct MomArgs {
     int nx, ny, nz;
+    int seg;                   // cells of a row in one task (a multiple of 16)
     double h3[2];              // cell volume, as a pair
     double org[3];             // the integer half cell nearest the origin, counted from the grid's corner, per axis
     double off[3][2];          // offset of that half cell from the origin in half cells (at most 1/2), as a pair
@@ -165,9 +166,12 @@ __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restri
     __shared__ double wm[kMomWarps][NB * 32][2], tot[NM][2], moved[NM][2];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int m = lane; m < NB * 32; m += 32) wm[warp][m][0] = wm[warp][m][1] = 0.0;
-    // tasks: (32 rows, 1 plane), plane fastest; a warp takes a contiguous range, so that its rows stay the same
-    const long long tasks = (long long)((P.ny + 31) / 32) * P.nz, W = (long long)kMomBlocks * kMomWarps;
-    const long long w = (long long)blockIdx.x * kMomWarps + warp;
+    // tasks: (segment of the rows, 32 rows, 1 plane), plane fastest; a warp takes a contiguous range, so that its rows stay the
+    // same.  Boxes of fewer than 32 rows put as many planes side by side in a task (nk) as the lanes hold.  Rows are cut into
+    // segments where there are fewer tasks than warps (mom_segment).
+    const int nk = P.ny < 32 ? 32 / P.ny : 1, dk = P.ny < 32 ? lane / P.ny : 0, dj = lane - dk * P.ny;  // lane -> plane, row
+    const int kt = (P.nz + nk - 1) / nk, jt = (P.ny + 31) / 32;
+    const long long W = (long long)kMomBlocks * kMomWarps, w = (long long)blockIdx.x * kMomWarps + warp;
     for (int x0 = 0; x0 < P.nx; x0 += ch) {
         const int x1 = P.nx < x0 + ch ? P.nx : x0 + ch;
         if constexpr (LMAX > 0) {
@@ -183,32 +187,35 @@ __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restri
             }
             __syncthreads();
         }
+        const long long tasks = (long long)((x1 - x0 + P.seg - 1) / P.seg) * jt * kt;
         long long t = w * tasks / W;
         const long long t1 = (w + 1) * tasks / W;
         while (t < t1) {
-            const int jg = (int)(t / P.nz), k0 = (int)(t % P.nz);
-            const int k1 = (int)(t1 - t < P.nz - k0 ? k0 + (t1 - t) : P.nz);
+            const long long part = t / kt;  // segment and rows
+            const int k0 = (int)(t - part * kt), k1 = (int)(t1 - t < kt - k0 ? k0 + (t1 - t) : kt);
             t += k1 - k0;
-            const int j = jg * 32 + lane;
-            const bool mine = j < P.ny;
+            const int s0 = x0 + (int)(part / jt) * P.seg, s1 = s0 + P.seg < x1 ? s0 + P.seg : x1;
+            const int j = (int)(part % jt) * 32 + dj;
             double As[LMAX + 1][LMAX + 1], Ae[LMAX + 1][LMAX + 1];  // [a][c], a + c <= LMAX
 #pragma unroll
             for (int a = 0; a <= LMAX; ++a)
 #pragma unroll
                 for (int c = 0; c <= LMAX; ++c) As[a][c] = Ae[a][c] = 0.0;
-            for (int k = k0; k < k1; ++k) {
-                const T* row = rho + ((long long)k * P.ny + (mine ? j : 0)) * P.nx;
-                const int hi = mine ? x1 : 0;
+            for (int kk = k0; kk < k1; ++kk) {
+                const int k = kk * nk + dk;
+                const bool mine = j < P.ny && dk < nk && k < P.nz;
+                const T* row = rho + (mine ? (long long)k * P.ny + j : 0ll) * P.nx;
+                const int hi = mine ? s1 : 0;
                 double Ts[LMAX + 1], Te[LMAX + 1];
 #pragma unroll
                 for (int a = 0; a <= LMAX; ++a) Ts[a] = Te[a] = 0.0;
                 T nv[kMomGroup];  // the next group's cells: in flight while this one is worked on
-                mom_load(row, x0, hi, vec, nv);
-                for (int i = x0; i < x1; i += kMomGroup) {
+                mom_load(row, s0, hi, vec, nv);
+                for (int i = s0; i < s1; i += kMomGroup) {
                     T v[kMomGroup];
 #pragma unroll
                     for (int e = 0; e < kMomGroup; ++e) v[e] = nv[e];
-                    if (i + kMomGroup < x1) mom_load(row, i + kMomGroup, hi, vec, nv);
+                    if (i + kMomGroup < s1) mom_load(row, i + kMomGroup, hi, vec, nv);
                     bool any = false;
 #pragma unroll
                     for (int e = 0; e < kMomGroup; ++e) any = any || nonzero(v[e]);
@@ -352,13 +359,25 @@ __global__ void __launch_bounds__(32) k_finish_moments(const double* __restrict_
     if (threadIdx.x == 0) out[blockIdx.x] = s;
 }
 
+// Cells of a row in one task: whole rows where those make a task for every warp, else equal parts of at least 128 cells (with
+// 64, 128^3 paid 133 us for a second Y^b and warp reduction against 117).  Float density, a call, us, for harmonics per cell
+// (whose threads do not care about the shape), whole rows of one plane per task, and this: lmax 0: 512 x 4 x 512 45, 84, 34;
+// 1024 x 1 x 1024 45, 207, 35; 2100 x 5 x 300 90, 272, 52; lmax 4: 900, 294, 114; 901, 778, 116; 2047, 991, 224.  Cubes from 224^3 on
+// have enough rows and are as they were.
+inline int mom_segment(int nx, int ny, int nz) {
+    const long long nk = ny < 32 ? 32 / ny : 1, rows = ((nz + nk - 1) / nk) * ((ny + 31) / 32), all = kMomBlocks * kMomWarps;
+    const long long parts = rows >= all ? 1 : all / rows;
+    const long long len = (nx + parts - 1) / parts;
+    return (int)((len > 128 ? len : 128) + kMomGroup - 1) & -kMomGroup;
+}
+
 // launch both kernels: the moments of rho (dense, device memory) into Q (device); scratch holds 2 kMomBlocks nq doubles
 template <int LMAX>
 cudaError_t launch_moments(const void* rho, int dtype, int nx, int ny, int nz, double h, const double* o, const YlmNorm& N,
                            double* scratch, double* Q, cudaStream_t st) {
     constexpr int NQ = (LMAX + 1) * (LMAX + 1);
     MomArgs P;
-    P.nx = nx, P.ny = ny, P.nz = nz;
+    P.nx = nx, P.ny = ny, P.nz = nz, P.seg = mom_segment(nx, ny, nz);
     const double h2 = h * h, h2e = fma(h, h, -h2);
     P.h3[0] = h2 * h;
     P.h3[1] = fma(h2, h, -P.h3[0]) + h2e * h;

@@ -95,3 +95,12 @@ def test_boxes_with_a_long_axis(lmax, shape):
     h = 1.0 / 48
     origin = tuple(-0.6 * n * h for n in shape)
     check(I.noise(shape[::-1], 412, 0.5, 1.5), h, origin, lmax, np.float64)
+
+
+@pytest.mark.parametrize("shape", [(140, 20, 7), (300, 40, 3), (520, 16, 5), (270, 1, 40), (129, 3, 23), (40, 31, 5)])
+@pytest.mark.parametrize("lmax", [0, 1, 4, 8])
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_thin_boxes(dtype, lmax, shape):
+    """Several planes of few rows in one task, and rows cut into segments where there are fewer tasks than warps."""
+    h = 1.0 / 32
+    check(I.noise(shape[::-1], 413, 0.5, 1.5), h, tuple(-0.45 * n * h for n in shape), lmax, dtype)
