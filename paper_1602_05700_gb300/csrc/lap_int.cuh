@@ -226,6 +226,7 @@ __host__ __device__ __forceinline__ double pack_units(long long S, unsigned h) {
     return A == 0 ? 0.0 : bits_d(top + mant);
 }
 
+// The next two are entry points of the host checks only (the sub-steps vote on a form per warp, cell.cuh).
 // L from integers; false when the stencil is left to FP64 (then L is not set)
 __host__ __device__ __forceinline__ bool lap6_int(double c, double x0, double x1, double x2, double x3, double x4,
                                                   double x5, double& L) {
