@@ -6,7 +6,8 @@
 // sub-steps that follow).  r^l Y_lm is a homogeneous polynomial with integer coefficients up to one factor, so the sums can
 // be taken axis by axis and the harmonics formed once per block:
 //   * a lane owns a row (fixed j, k), or a part of one, and sums rho X^a over it, four cells at a time in plain FP64 and from there on in
-//     double-double (T_a): 9 operations per cell at lmax = 4.  X is the same for all lanes, so its powers come from a table in
+//     double-double (T_a; the rounding error of one addition starts the next four cells' sum): 9 operations per cell at lmax =
+//     4.  X is the same for all lanes, so its powers come from a table in
 //     shared memory, each rounded once;
 //   * T_a times Z^c goes to the lane's sums over k (10 per row and (a, c)); Y^b, a transposing warp reduction (31 merges
 //     per 32 moments), the sum over warps and the change to Q_lm follow once per block.  Y^b and Z^c are pairs.
@@ -20,8 +21,9 @@
 // source) are skipped.
 //
 // Measured (random density, a call of hg_moments_noalloc with both its launches, us, harmonics per cell -> this): lmax 4:
-// 32^3 347 -> 74, 128^3 1475 -> 117, 256^3 9490 -> 449, 512^3 73,500 -> 2790; lmax 8: 256^3 30,030 -> 925; lmax 0: 256^3 374 ->
-// 116.  (Sums of 16 cells in plain FP64 about the grid's centre: 407 at 256^3 and lmax 4.)  Error in units of 2^-53 sum |rho| |x|^l
+// 32^3 347 -> 73, 128^3 1475 -> 114, 256^3 9490 -> 413, 512^3 73,500 -> 2500; lmax 8: 256^3 30,030 -> 852; lmax 0: 256^3 374 ->
+// 116.  (With the errors summed beside T_a: 449 at 256^3 and lmax 4; sums of 16 cells in plain FP64 about the grid's
+// centre: 407, 512^3 2083.)  Error in units of 2^-53 sum |rho| |x|^l
 // over spheres, Gaussians, constants and noise, centred or up to 0.8 of the way to a face, lmax 4 and 8 (the kernel's order
 // evaluated on the host against quad precision; harmonics per cell with an exact sum -> this): largest 0.74 -> 0.44.
 #pragma once
@@ -74,15 +76,16 @@ static __device__ const HarmonicTable kHarmonics = make_harmonics();
 // rounding error that the lossless scheme then carries, through the Dirichlet data, into phi; so every partial sum
 // is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding errors), whose
 // error is of order n eps^2 of the sum of |terms|.
-// TwoSum as FastTwoSum on the operands ordered by the high words of their magnitudes (so the first one's exponent is not the
-// smaller): three FP64 operations and integer selects, where TwoSum takes six on the pipe that bounds the kernel.
-__device__ __forceinline__ void dd_add(double& s, double& e, double x) {
+// s <- s + x, and its rounding error: TwoSum as FastTwoSum on the operands ordered by the high words of their magnitudes (so the
+// first one's exponent is not the smaller): three FP64 operations and integer selects, where TwoSum takes six on the pipe that
+// bounds the kernel.
+__device__ __forceinline__ double sum_error(double& s, double x) {
     const bool swap = (__double2hiint(s) & 0x7fffffff) < (__double2hiint(x) & 0x7fffffff);
     const double a = swap ? x : s, b = swap ? s : x;
-    const double t = __dadd_rn(a, b);
-    e = __dadd_rn(e, __dsub_rn(b, __dsub_rn(t, a)));
-    s = t;
+    s = __dadd_rn(a, b);
+    return __dsub_rn(b, __dsub_rn(s, a));
 }
+__device__ __forceinline__ void dd_add(double& s, double& e, double x) { e = __dadd_rn(e, sum_error(s, x)); }
 // (s, e) += (s2, e2), renormalised so that s is the rounded value of the pair
 __device__ __forceinline__ void dd_merge(double& s, double& e, double s2, double e2) {
     dd_add(s, e, s2);
@@ -229,13 +232,13 @@ __global__ void __launch_bounds__(32 * kMomWarps, 1) k_moments(const T* __restri
                         for (int a = 0; a <= LMAX; ++a) {
                             double s;
                             if (a == 0) {
-                                s = __dadd_rn(__dadd_rn(c[0], c[1]), __dadd_rn(c[2], c[3]));
+                                s = __dadd_rn(__dadd_rn(__dadd_rn(Te[a], c[0]), c[1]), __dadd_rn(c[2], c[3]));
                             } else {
                                 const double2* p = reinterpret_cast<const double2*>(pw + (a - 1) * ch + (i - x0 + g));
                                 const double2 pa = p[0], pb = p[1];
-                                s = __fma_rn(c[3], pb.y, __fma_rn(c[2], pb.x, __fma_rn(c[1], pa.y, __dmul_rn(c[0], pa.x))));
+                                s = __fma_rn(c[3], pb.y, __fma_rn(c[2], pb.x, __fma_rn(c[1], pa.y, __fma_rn(c[0], pa.x, Te[a]))));
                             }
-                            dd_add(Ts[a], Te[a], s);
+                            Te[a] = sum_error(Ts[a], s);  // goes into the next four cells' sum
                         }
                     }
                 }
@@ -361,8 +364,8 @@ __global__ void __launch_bounds__(32) k_finish_moments(const double* __restrict_
 
 // Cells of a row in one task: whole rows where those make a task for every warp, else equal parts of at least 128 cells (with
 // 64, 128^3 paid 133 us for a second Y^b and warp reduction against 117).  Float density, a call, us, for harmonics per cell
-// (whose threads do not care about the shape), whole rows of one plane per task, and this: lmax 0: 512 x 4 x 512 45, 84, 34;
-// 1024 x 1 x 1024 45, 207, 35; 2100 x 5 x 300 90, 272, 52; lmax 4: 900, 294, 114; 901, 778, 116; 2047, 991, 224.  Cubes from 224^3 on
+// (whose threads do not care about the shape), whole rows of one plane per task, and this: lmax 0: 512 x 4 x 512 45, 84, 35;
+// 1024 x 1 x 1024 45, 207, 36; 2100 x 5 x 300 90, 272, 52; lmax 4: 900, 294, 110; 901, 778, 113; 2047, 991, 215.  Cubes from 224^3 on
 // have enough rows and are as they were.
 inline int mom_segment(int nx, int ny, int nz) {
     const long long nk = ny < 32 ? 32 / ny : 1, rows = ((nz + nk - 1) / nk) * ((ny + 31) / 32), all = kMomBlocks * kMomWarps;
