@@ -134,7 +134,8 @@ int hg_set_temporal_exact(hg_grid* g, int exact);
 
 /* z planes per thread block of the compensated-float single sweep's z-marching kernel (a tuning knob: more blocks and
  * more z warm-up below, fewer and longer blocks above); 0 restores the built-in rule, under which small grids do not march
- * at all.  FP64 sub-steps never march.  Results do not depend on it. */
+ * at all.  FP64 sub-steps never march; the fused depth-2 kernel takes at most 32 planes; batches choose their
+ * own and the adjoint keeps the built-in rule.  Results do not depend on it. */
 int hg_set_block_depth(hg_grid* g, int planes);
 
 /*

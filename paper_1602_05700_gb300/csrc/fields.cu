@@ -456,7 +456,7 @@ inline unsigned cells_blocks(const hg_grid* g) {
 
 template <typename TS, typename TD, bool SUM, bool MEAN>
 static void pack_launch(hg_grid* g, const void* src) {
-    // the narrower of the two types sets the group: 16 bytes of it
+    // the wider of the two types sets the group: 16 bytes of it
     using T = std::conditional_t<(sizeof(TS) < sizeof(TD)), TD, TS>;
     dispatch_groups<T>(g->L, dense_width<T>(g->L, {src}), [&](auto W, auto I) {
         const unsigned blocks = SUM ? (unsigned)kPackBlocks : group_blocks(g->L, W);

@@ -134,10 +134,12 @@ int ensure_hydro_staging(hg_hydro* H) {
     return HG_OK;
 }
 
-// z planes per block.  FP32: about 2800 blocks, at least 8 planes each (280^3: 765 us per stage with 74 planes, 716 with
-// 32, 760 with 8).  FP64: the pipe of each SM is the bound, so the planes go out as evenly over the SMs as chunks of 6 to
-// 16 allow; a block's start-up is worth 0.9 planes (96^3: 12 planes, 288 blocks, 1782 us against 1845 with 8, 432 blocks;
-// 140^3: 14 planes 6059 against 6296 with 11; measured before the integer comparisons).
+// z planes per block.  FP32: about 2800 blocks, at least 8 planes each.  Us per stage, this rule -> the best of 4 to 64 planes:
+// 64^3 20.4 -> 18.3 (4), 96^3 38.1 -> 38.7, 140^3 119.7 -> 113.7 (28), 200^3 301 -> 288 (32), 240^3 468 -> 469, 280^3 712 -> 707 (24; 753
+// with 8), 301x259x223 602 -> 588 (40), 400^3 2069 -> 2007 (64).  FP64: the pipe of each SM is the bound, so the planes go out as
+// evenly over the SMs as chunks of 6 to 16 allow; a block's start-up is worth 0.9 planes.  This rule -> the best of 5 to 20:
+// 48^3 403 -> 341 (5), 64^3 524 -> 524, 96^3 1430 -> 1431 (12; 1492 with 8), 120^3 2858 -> 2859, 140^3 4959 -> 4960 (14; 5207 with 11),
+// 200^3 13,656 -> 13,653 (16), 97x83x61 1318 -> 1206 (10).
 int stage_zb(const hg_hydro* H) {
     const long long nxy = (long long)((H->nx + TX - 1) / TX) * ((H->ny + TY - 1) / TY);
     long long zb = 0;

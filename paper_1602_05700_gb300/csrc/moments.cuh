@@ -5,10 +5,10 @@
 // a double-double sum costs about 240 FP64 operations per cell at lmax = 4 (9.3 ms at 256^3, against 1.5 ms for the 20
 // sub-steps that follow).  r^l Y_lm is a homogeneous polynomial with integer coefficients up to one factor, so the sums can
 // be taken axis by axis and the harmonics formed once per block:
-//   * a lane owns a row (fixed j, k), or a part of one, and sums rho X^a over it, four cells at a time in plain FP64 and from there on in
-//     double-double (T_a; the rounding error of one addition starts the next four cells' sum): 9 operations per cell at lmax =
-//     4.  X is the same for all lanes, so its powers come from a table in
-//     shared memory, each rounded once;
+//   * a lane owns a row (fixed j, k), or a part of one, and sums rho X^a over it, four cells at a time in plain FP64 and from
+//     there on in double-double (T_a; the rounding error of one addition starts the next four cells' sum): 9 operations
+//     per cell at lmax = 4.  X is the same for all lanes, so its powers come from a table in shared memory, each rounded
+//     once;
 //   * T_a times Z^c goes to the lane's sums over k (10 per row and (a, c)); Y^b, a transposing warp reduction (31 merges
 //     per 32 moments), the sum over warps and the change to Q_lm follow once per block.  Y^b and Z^c are pairs.
 // Coordinates are half cells counted from the integer one nearest the expansion origin, so a term is no larger than the moment
@@ -23,9 +23,9 @@
 // Measured (random density, a call of hg_moments_noalloc with both its launches, us, harmonics per cell -> this): lmax 4:
 // 32^3 347 -> 73, 128^3 1475 -> 114, 256^3 9490 -> 413, 512^3 73,500 -> 2500; lmax 8: 256^3 30,030 -> 852; lmax 0: 256^3 374 ->
 // 116.  (With the errors summed beside T_a: 449 at 256^3 and lmax 4; sums of 16 cells in plain FP64 about the grid's
-// centre: 407, 512^3 2083.)  Error in units of 2^-53 sum |rho| |x|^l
-// over spheres, Gaussians, constants and noise, centred or up to 0.8 of the way to a face, lmax 4 and 8 (the kernel's order
-// evaluated on the host against quad precision; harmonics per cell with an exact sum -> this): largest 0.74 -> 0.44.
+// centre: 407, 512^3 2083.)  Error in units of 2^-53 sum |rho| |x|^l over spheres, Gaussians, constants and noise, centred or up
+// to 0.8 of the way to a face, lmax 4 and 8 (the kernel's order evaluated on the host against quad precision; harmonics per
+// cell with an exact sum -> this): largest 0.74 -> 0.44.
 #pragma once
 
 #include "cell.cuh"
@@ -74,8 +74,8 @@ static __device__ const HarmonicTable kHarmonics = make_harmonics();
 // ---- double-double sums --------------------------------------------------------------------------------------
 // Each moment is a sum over every cell (1.7e7 terms at 256^3).  A plain running or tree sum in FP64 carries a
 // rounding error that the lossless scheme then carries, through the Dirichlet data, into phi; so every partial sum
-// is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding errors), whose
-// error is of order n eps^2 of the sum of |terms|.
+// beyond four cells is kept as an unevaluated pair s + e (TwoSum: s is the rounded sum, e collects the exact rounding
+// errors), whose error is of order n eps^2 of the sum of |terms|.
 // s <- s + x, and its rounding error: TwoSum as FastTwoSum on the operands ordered by the high words of their magnitudes (so the
 // first one's exponent is not the smaller): three FP64 operations and integer selects, where TwoSum takes six on the pipe that
 // bounds the kernel.

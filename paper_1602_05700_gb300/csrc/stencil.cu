@@ -25,7 +25,9 @@ namespace {
 constexpr int kWY = 8;
 
 // z planes per block of the TMA-staged sweep: short chunks, many blocks -- the stage ring hides the z warm-up, and fine
-// blocks balance the SMs (measured at 512^3: 8 planes beat 16-64)
+// blocks balance the SMs, also where the last wave is nearly empty.  Us per sub-step (Robin) with 8 planes, the best of 6 to 48,
+// and 25: 230^3 62.4, 62.3 (6), 83.1; 256^3 77.7, 76.8 (6), 92.1; 301x259x223 83.3, 83.2 (12), 91.8; 320^3 142.3, 141.5 (12), 152.2;
+// 360^3 186.3, 186.3, 201.6; 400^3 264.2, 258.8 (12), 270.4; 512x256x128 73.5, 72.2 (6), 88.6; 512^3 497, 494 (6), 526.
 int zchunk(const hg_grid* g) { return g->nz < 8 ? g->nz : 8; }
 
 // entry of block b in a prefix table of n entries (first[0] = 0): 32 at a time, every lane one

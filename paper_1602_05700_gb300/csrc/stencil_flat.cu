@@ -21,12 +21,14 @@ namespace {
 
 constexpr int kFlatThreads = 128;
 
-// FP64: two cells per thread from here on.  They share the conversions of the integer forms (198 instructions per cell
+// FP64: two cells per thread from here on.  They share the conversions of the integer forms (194 instructions per cell
 // instead of 248) and move 16 bytes per access; smaller grids want the threads.  Measured, us per sub-step, one -> two cells:
 // 32^3 2.59 -> 4.1, 64^3 4.82 -> 4.82, 96^3 10.9 -> 10.5, 128^3 22.6 -> 20.6, 192^3 75.4 -> 67.4, 256^3 176 -> 155,
 // 301x259x223 184 -> 165.  (Marching 2 to 16 planes per thread, with or without square tiles, 144-150 us in a field where this
-// takes 148: the loads it saves do not bound it.)  The adjoint's reverse sub-steps keep one cell per thread: their injection is
-// sparse, and a warp of 64 cells is oftener left to FP64 (128^3 adjoint 10.6 against 11.2 ms).
+// takes 148: the loads it saves do not bound it.)  The adjoint's reverse sub-steps keep one cell per thread: lambda changes sign, and
+// a warp of 64 cells is oftener left to FP64.  Us per reverse sub-step, one -> two cells: 64 injected cells 96^3 29.0 -> 29.5, 128^3
+// 61.0 -> 63.4, 192^3 180 -> 190, 256^3 370 -> 398; noise in every cell 30.5 -> 30.3, 68.2 -> 68.3, 223 -> 223, 523 -> 521; only a smooth
+// injection of one sign gains, 12.6 -> 13.8, 25.2 -> 25.9, 90.6 -> 84.7, 209 -> 192.
 constexpr long long kPairCells = 600000;
 
 template <bool ADJ, bool WIDE>

@@ -541,10 +541,11 @@ int launch_temporal2_tma(hg_grid* g) {
     A.B.periodic = 0;
     const int c = g->cur;
     dim3 grid((g->nx + kFX - 1) / kFX, (g->ny + kFY - 1) / kFY, (g->nz + zb - 1) / zb);
-    // which code (see fused2_block).  Whole tiles where nx allows them (320^3 139 against 173 us per sub-step, 512^3 422
-    // against 471 before the copies went first), except in exact mode on grids of more than one wave of blocks, where the general code comes out
-    // faster (512^3: 483 against 521 us; the register allocation of the scalar update differs), not on smaller ones
-    // (128^3: 32 against 37)
+    // which code (see fused2_block).  Whole tiles where nx allows them (320^3 137 against 173 us per sub-step), except in exact
+    // mode on grids of more than one wave of blocks (304): there the register allocation of the scalar update differs, and
+    // the general code is the faster one for the large grids that fused sub-steps are for.  Exact mode, us per sub-step,
+    // general -> whole tiles, Robin and Dirichlet: 128^3 37 -> 33 (Robin), 224^3 86 -> 75, 67 -> 67.5; 256^3 84.7 -> 82.4, 68.5 -> 71.3;
+    // 320^3 175 -> 166, 145 -> 143; 384^3 217 -> 232, 198 -> 208; 512^3 476 -> 516, 443 -> 473.
     const bool whole = g->nx >= kFX && g->nx % 8 == 0 && !(g->texact && (long long)grid.x * grid.y * grid.z > 304);
     const int v = (!whole ? 0 : g->nx % kFX == 0 ? 1 : 2) + (g->texact ? 3 : 0);
     static unsigned long long attr_done[6] = {0, 0, 0, 0, 0, 0};
