@@ -406,8 +406,11 @@ cudaError_t launch_moments(const void* rho, int dtype, int nx, int ny, int nz, d
     constexpr int NM = mono_off(LMAX + 1), held = 16 * (kMomWarps * ((NM + 31) / 32) * 32 + 2 * NM);  // static part
     cudaError_t e = cudaSuccess;
     auto launch = [&](auto* kernel, const auto* r) {
-        if (held + smem > 48 * 1024)  // above 48 KB a kernel has to ask (each time: a device reset forgets it)
-            e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        // above 48 KB a kernel has to ask: each time, as a device reset forgets it, and always for the most, as another host
+        // thread may be about to launch it for longer rows
+        if (held + smem > 48 * 1024)
+            e = cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     LMAX * kMomStretch * (int)sizeof(double));
         if (e != cudaSuccess) return;
         kernel<<<kMomBlocks, th, smem, st>>>(r, vec, P, N, scratch, ch);
         e = cudaGetLastError();

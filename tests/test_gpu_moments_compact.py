@@ -5,6 +5,7 @@ The rounding error has to scale with the source's own extent about the origin, n
 |x| + h/2, |y| + h/2, |z| + h/2 (the kernel counts half cells from the one nearest the origin) in the absolute value of
 every term of r^l Y_lm.  Roundings per term, each 2^-53 of it: the power (1), the product and the sum of four cells (4), the
 normalisation (2), the result (1); everything else is carried in pairs: 8 in all."""
+from concurrent.futures import ThreadPoolExecutor
 from math import factorial
 
 import numpy as np
@@ -104,3 +105,22 @@ def test_thin_boxes(dtype, lmax, shape):
     """Several planes of few rows in one task, and rows cut into segments where there are fewer tasks than warps."""
     h = 1.0 / 32
     check(I.noise(shape[::-1], 413, 0.5, 1.5), h, tuple(-0.45 * n * h for n in shape), lmax, dtype)
+
+
+def test_threads_with_rows_of_different_lengths():
+    """The table of powers takes shared memory by the row's length; grids of short and long rows share the kernel."""
+    def moments_of(nx, times):
+        g = hg.Grid(nx, 3, 2, 1.0 / 32, (-1.0, 0.0, 0.0), 1.0, 1.0, 1.0 / 128, "f64", "multipole", 8)
+        rho = torch.from_numpy(I.noise((2, 3, nx), 414, 0.5, 1.5)).cuda()
+        out = []
+        for _ in range(times):
+            g.set_density(rho)
+            out.append(g.moments())
+        g.free()
+        return np.array(out)
+
+    lengths = [2000, 320, 900, 2100]
+    alone = {nx: moments_of(nx, 1)[0] for nx in lengths}
+    with ThreadPoolExecutor(len(lengths)) as ex:
+        for nx, out in zip(lengths, ex.map(lambda nx: moments_of(nx, 40), lengths)):
+            assert (out == alone[nx]).all()
